@@ -61,11 +61,14 @@ __device__ __forceinline__ f2 operator-(const f2p& p, const f2p& q) {
 __device__ __forceinline__ f2& operator+=(f2& a, const f2& b) { return a = a + b; }
 __device__ __forceinline__ f2& operator-=(f2& a, const f2& b) { return a = a - b; }
 
+__device__ __forceinline__ f2 mad(const f2& a, const f2& b, const f2& c) { return f2(__ffma2_rn(a.v, b.v, c.v)); }
+
 // Per-lane operations without a packed form.
 __device__ __forceinline__ f2 fdiv(const f2& a, const f2& b) {
     return f2(make_float2(__fdividef(a.v.x, b.v.x), __fdividef(a.v.y, b.v.y)));
 }
-__device__ __forceinline__ f2 sqrt(const f2& a) { return f2(make_float2(sqrtf(a.v.x), sqrtf(a.v.y))); }
+__device__ __forceinline__ f2 recip(const f2& b) { return fdiv(f2(1.0f), b); }
+__device__ __forceinline__ f2 root(const f2& a) { return f2(make_float2(sqrtf(a.v.x), sqrtf(a.v.y))); }
 
 __device__ __forceinline__ f2 cs_dev(const f2& b, const f2& rho0, const f2& Rg, const f2& rho_d, const f2& T,
                                      const f2& T_d) {

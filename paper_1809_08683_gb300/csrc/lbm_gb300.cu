@@ -598,36 +598,32 @@ __global__ void __launch_bounds__(BX, KEEP ? FusedTraits<R, BX>::MINB : FusedTra
         issue(k + S);  // stage of logical row k is free: its collision finished before the barrier
 
         if (active) {
-            if (KEEP && !(isfinite(mc.rho_d) && isfinite(mc.T_d))) atomicOr(status, 1u);
+            if (KEEP && !(lbm::finite(mc.rho_d) && lbm::finite(mc.T_d))) atomicOr(status, 1u);
             // ring slots of the rows j - 1 (sm), j, j + 1 (sp)
             const int sm = (down ? k + 2 : k) & 3, s0 = (k + 1) & 3, sp = (down ? k : k + 2) & 3;
             const bool onS = !py && j == 0, onN = !py && j == ny - 1;
             const bool onW = !px && x == 0, onE = !px && x == nx - 1;
             R grx, gry, gpx, gpy;
             if (!(onS || onN || onW || onE)) {
-                // grad = 3 sum_i w_i e_i phi(x + e_i), w = 1/9 (axis), 1/36 (diagonal)
-                const R t = R(1.0 / 3.0), d = R(1.0 / 12.0);
                 const RhoP<R> ml = s_rp[sm][c - 1], mc_ = s_rp[sm][c], mr = s_rp[sm][c + 1];
                 const RhoP<R> zl = s_rp[s0][c - 1], zr = s_rp[s0][c + 1];
                 const RhoP<R> pl = s_rp[sp][c - 1], pc = s_rp[sp][c], pr = s_rp[sp][c + 1];
-                grx = t * (zr.r - zl.r) + d * ((pr.r - pl.r) + (mr.r - ml.r));
-                gry = t * (pc.r - mc_.r) + d * ((pr.r - mr.r) + (pl.r - ml.r));
-                gpx = t * (zr.p - zl.p) + d * ((pr.p - pl.p) + (mr.p - ml.p));
-                gpy = t * (pc.p - mc_.p) + d * ((pr.p - mr.p) + (pl.p - ml.p));
+                lbm::gradient3(ml.r, mc_.r, mr.r, zl.r, zr.r, pl.r, pc.r, pr.r, grx, gry);
+                lbm::gradient3(ml.p, mc_.p, mr.p, zl.p, zr.p, pl.p, pc.p, pr.p, gpx, gpy);
             } else {
                 // wall node: one-sided second order along the inward normal,
-                // central along the wall
+                // central along the wall (three times each, as gradient3)
                 const R r0 = s_rp[s0][c].r, p0 = s_rp[s0][c].p;
                 if (onW || onE) {
                     const int dx = onW ? 1 : -1;
                     R r2, p2;
                     rho_p_at<MC>(P, src, plane, pitch, x + 2 * dx, j, r2, p2);
                     const R r1 = s_rp[s0][c + dx].r, p1 = s_rp[s0][c + dx].p;
-                    grx = R(dx) * (R(-3) * r0 + R(4) * r1 - r2) * R(0.5);
-                    gpx = R(dx) * (R(-3) * p0 + R(4) * p1 - p2) * R(0.5);
+                    grx = R(dx) * (R(-3) * r0 + R(4) * r1 - r2) * R(1.5);
+                    gpx = R(dx) * (R(-3) * p0 + R(4) * p1 - p2) * R(1.5);
                 } else {
-                    grx = (s_rp[s0][c + 1].r - s_rp[s0][c - 1].r) * R(0.5);
-                    gpx = (s_rp[s0][c + 1].p - s_rp[s0][c - 1].p) * R(0.5);
+                    grx = (s_rp[s0][c + 1].r - s_rp[s0][c - 1].r) * R(1.5);
+                    gpx = (s_rp[s0][c + 1].p - s_rp[s0][c - 1].p) * R(1.5);
                 }
                 if (onS || onN) {
                     const int dy = onS ? 1 : -1;
@@ -635,11 +631,11 @@ __global__ void __launch_bounds__(BX, KEEP ? FusedTraits<R, BX>::MINB : FusedTra
                     rho_p_at<MC>(P, src, plane, pitch, x, j + 2 * dy, r2, p2);
                     const R r1 = onS ? s_rp[sp][c].r : s_rp[sm][c].r;
                     const R p1 = onS ? s_rp[sp][c].p : s_rp[sm][c].p;
-                    gry = R(dy) * (R(-3) * r0 + R(4) * r1 - r2) * R(0.5);
-                    gpy = R(dy) * (R(-3) * p0 + R(4) * p1 - p2) * R(0.5);
+                    gry = R(dy) * (R(-3) * r0 + R(4) * r1 - r2) * R(1.5);
+                    gpy = R(dy) * (R(-3) * p0 + R(4) * p1 - p2) * R(1.5);
                 } else {
-                    gry = (s_rp[sp][c].r - s_rp[sm][c].r) * R(0.5);
-                    gpy = (s_rp[sp][c].p - s_rp[sm][c].p) * R(0.5);
+                    gry = (s_rp[sp][c].r - s_rp[sm][c].r) * R(1.5);
+                    gpy = (s_rp[sp][c].p - s_rp[sm][c].p) * R(1.5);
                 }
             }
 
@@ -652,7 +648,7 @@ __global__ void __launch_bounds__(BX, KEEP ? FusedTraits<R, BX>::MINB : FusedTra
                 lbm::expand<MC>(P, mc, mf);
             } else {
                 node_macros<MC>(P, v, mf);
-                if (!(isfinite(mf.rho_d) && isfinite(mf.T_d))) atomicOr(status, 1u);
+                if (!(lbm::finite(mf.rho_d) && lbm::finite(mf.T_d))) atomicOr(status, 1u);
             }
             AddDither add(mix32(step_hash ^ ((uint32_t)j * 0x85ebca77u + (uint32_t)x * 0xc2b2ae3du)), dscale);
             // block strips keep the DFs in registers through the collision
@@ -858,17 +854,13 @@ __global__ void __launch_bounds__(32 * NW, WarpTraits<R>::WARPS_PER_SM / NW)
         const R p0l = __shfl_up_sync(FULL, p0, 1), p0r = __shfl_down_sync(FULL, p0, 1);
         const R ppl = __shfl_up_sync(FULL, pp, 1), ppr = __shfl_down_sync(FULL, pp, 1);
         if (owned) {
-            if (!(isfinite(mc.rho_d) && isfinite(mc.T_d))) atomicOr(status, 1u);
+            if (!(lbm::finite(mc.rho_d) && lbm::finite(mc.T_d))) atomicOr(status, 1u);
             const bool onS = !py && j == 0, onN = !py && j == ny - 1;
             const bool onW = !px && x == 0, onE = !px && x == nx - 1;
             R grx, gry, gpx, gpy;
             if (!(onS || onN || onW || onE)) {
-                // grad = 3 sum_i w_i e_i phi(x + e_i), w = 1/9 (axis), 1/36 (diagonal)
-                const R t = R(1.0 / 3.0), d = R(1.0 / 12.0);
-                grx = t * (r0r - r0l) + d * ((rpr - rpl) + (rmr - rml));
-                gry = t * (rp - rm) + d * ((rpr - rmr) + (rpl - rml));
-                gpx = t * (p0r - p0l) + d * ((ppr - ppl) + (pmr - pml));
-                gpy = t * (pp - pm) + d * ((ppr - pmr) + (ppl - pml));
+                lbm::gradient3(rml, rm, rmr, r0l, r0r, rpl, rp, rpr, grx, gry);
+                lbm::gradient3(pml, pm, pmr, p0l, p0r, ppl, pp, ppr, gpx, gpy);
             } else {
                 // wall node: one-sided second order along the inward normal,
                 // central along the wall
@@ -877,22 +869,22 @@ __global__ void __launch_bounds__(32 * NW, WarpTraits<R>::WARPS_PER_SM / NW)
                     R r2, p2;
                     rho_p_at<MC>(P, src, plane, pitch, x + 2 * dx, j, r2, p2);
                     const R r1 = onW ? r0r : r0l, p1 = onW ? p0r : p0l;
-                    grx = R(dx) * (R(-3) * r0 + R(4) * r1 - r2) * R(0.5);
-                    gpx = R(dx) * (R(-3) * p0 + R(4) * p1 - p2) * R(0.5);
+                    grx = R(dx) * (R(-3) * r0 + R(4) * r1 - r2) * R(1.5);
+                    gpx = R(dx) * (R(-3) * p0 + R(4) * p1 - p2) * R(1.5);
                 } else {
-                    grx = (r0r - r0l) * R(0.5);
-                    gpx = (p0r - p0l) * R(0.5);
+                    grx = (r0r - r0l) * R(1.5);
+                    gpx = (p0r - p0l) * R(1.5);
                 }
                 if (onS || onN) {
                     const int dy = onS ? 1 : -1;
                     R r2, p2;
                     rho_p_at<MC>(P, src, plane, pitch, x, j + 2 * dy, r2, p2);
                     const R r1 = onS ? rp : rm, p1 = onS ? pp : pm;
-                    gry = R(dy) * (R(-3) * r0 + R(4) * r1 - r2) * R(0.5);
-                    gpy = R(dy) * (R(-3) * p0 + R(4) * p1 - p2) * R(0.5);
+                    gry = R(dy) * (R(-3) * r0 + R(4) * r1 - r2) * R(1.5);
+                    gpy = R(dy) * (R(-3) * p0 + R(4) * p1 - p2) * R(1.5);
                 } else {
-                    gry = (rp - rm) * R(0.5);
-                    gpy = (pp - pm) * R(0.5);
+                    gry = (rp - rm) * R(1.5);
+                    gpy = (pp - pm) * R(1.5);
                 }
             }
 
@@ -952,9 +944,9 @@ struct PairSmem {
 __device__ void broadcast_params(const Params<float>& a, Params<f2>& b) {
 #define BP(f) b.f = f2(a.f)
     BP(rho0); BP(T0); BP(E0); BP(Cv); BP(inv_Cv); BP(Rg); BP(eos_a); BP(eos_b); BP(p0); BP(rho0E0_p0);
-    BP(rho0Cp0); BP(mu0); BP(inv_T0); BP(visc_S); BP(lam_fac); BP(tj_fac); BP(e_fac); BP(alpha1);
-    BP(beta1); BP(alpha2); BP(beta2); BP(kk); BP(hh); BP(bb); BP(gamma1); BP(gamma2); BP(cR11);
-    BP(cR17); BP(cR18); BP(cR71); BP(cR77); BP(cR81); BP(cR88); BP(Fx); BP(Fy); BP(cs_b0); BP(dither);
+    BP(rho0Cp0); BP(mu0); BP(mu0S); BP(inv_T0); BP(visc_S); BP(lam_fac); BP(nu_e); BP(mu_j); BP(beta2);
+    BP(kk); BP(hh); BP(bb); BP(omk); BP(k2h); BP(gamma1); BP(gamma2); BP(k11); BP(k17); BP(k18);
+    BP(k71); BP(k77); BP(k81); BP(k88); BP(Fx); BP(Fy); BP(cs_b0); BP(dither);
 #undef BP
     b.eos = a.eos;
     b.visc = a.visc;
@@ -1140,8 +1132,8 @@ __global__ void __launch_bounds__(BX / 2, (KEEP ? LBM_PAIR_WARPS_PER_SM : 12) * 
         issue(k + S);
 
         if (act_a) {
-            if (KEEP && !(isfinite(mc.rho_d.v.x) && isfinite(mc.T_d.v.x) && isfinite(mc.rho_d.v.y) && isfinite(mc.T_d.v.y)))
-                atomicOr(status, act_b ? 1u : ((isfinite(mc.rho_d.v.x) && isfinite(mc.T_d.v.x)) ? 0u : 1u));
+            if (KEEP && !(lbm::finite(mc.rho_d.v.x) && lbm::finite(mc.T_d.v.x) && lbm::finite(mc.rho_d.v.y) && lbm::finite(mc.T_d.v.y)))
+                atomicOr(status, act_b ? 1u : ((lbm::finite(mc.rho_d.v.x) && lbm::finite(mc.T_d.v.x)) ? 0u : 1u));
             // ring slots of the rows j - 1 (sm), j, j + 1 (sp)
             const int sm = (down ? k + 2 : k) & 3, s0 = (k + 1) & 3, sp = (down ? k : k + 2) & 3;
             // interior stencil for both nodes: columns (ca-1, ca) on the left, (ca+1, ca+2) on the right
@@ -1152,9 +1144,7 @@ __global__ void __launch_bounds__(BX / 2, (KEEP ? LBM_PAIR_WARPS_PER_SM : 12) * 
                 const f2 lm(make_float2(a[sm][ca - 1], cm.x)), rm(make_float2(cm.y, a[sm][ca + 2]));
                 const f2 l0(make_float2(a[s0][ca - 1], c0.x)), r0(make_float2(c0.y, a[s0][ca + 2]));
                 const f2 lp(make_float2(a[sp][ca - 1], cp.x)), rp(make_float2(cp.y, a[sp][ca + 2]));
-                const f2 t(1.0f / 3.0f), d(1.0f / 12.0f);
-                gx = t * (r0 - l0) + d * ((rp - lp) + (rm - lm));
-                gy = t * (f2(cp) - f2(cm)) + d * ((rp - rm) + (lp - lm));
+                lbm::gradient3(lm, f2(cm), rm, l0, r0, lp, f2(cp), rp, gx, gy);
             };
             f2 grx, gry, gpx, gpy;
             grad(s_rho, grx, gry);
@@ -1194,15 +1184,15 @@ __global__ void __launch_bounds__(BX / 2, (KEEP ? LBM_PAIR_WARPS_PER_SM : 12) * 
                         const float v0 = a[s0][c];
                         float gxs, gys;
                         if (onW || onE) {
-                            gxs = (float)dx * (-3.0f * v0 + 4.0f * a[s0][c + dx] - (fld ? px2 : rx2)) * 0.5f;
+                            gxs = (float)dx * (-3.0f * v0 + 4.0f * a[s0][c + dx] - (fld ? px2 : rx2)) * 1.5f;
                         } else {
-                            gxs = (a[s0][c + 1] - a[s0][c - 1]) * 0.5f;
+                            gxs = (a[s0][c + 1] - a[s0][c - 1]) * 1.5f;
                         }
                         if (onS || onN) {
                             const float v1 = onS ? a[sp][c] : a[sm][c];
-                            gys = (float)dy * (-3.0f * v0 + 4.0f * v1 - (fld ? py2 : ry2)) * 0.5f;
+                            gys = (float)dy * (-3.0f * v0 + 4.0f * v1 - (fld ? py2 : ry2)) * 1.5f;
                         } else {
-                            gys = (a[sp][c] - a[sm][c]) * 0.5f;
+                            gys = (a[sp][c] - a[sm][c]) * 1.5f;
                         }
                         gr[2 * fld] = gxs;
                         gr[2 * fld + 1] = gys;
@@ -1223,7 +1213,7 @@ __global__ void __launch_bounds__(BX / 2, (KEEP ? LBM_PAIR_WARPS_PER_SM : 12) * 
                 f2 rd, jx, jy, sg;
                 lbm::node_sums(v, v + 9, rd, jx, jy, sg);
                 lbm::macros<MC>(P2, rd, jx, jy, sg, mf);
-                if (!(isfinite(mf.rho_d.v.x) && isfinite(mf.T_d.v.x) && (!act_b || (isfinite(mf.rho_d.v.y) && isfinite(mf.T_d.v.y)))))
+                if (!(lbm::finite(mf.rho_d.v.x) && lbm::finite(mf.T_d.v.x) && (!act_b || (lbm::finite(mf.rho_d.v.y) && lbm::finite(mf.T_d.v.y)))))
                     atomicOr(status, 1u);
             }
             AddDither2 add(mix32(step_hash ^ ((uint32_t)j * 0x85ebca77u + (uint32_t)xa * 0xc2b2ae3du)), dscale);
@@ -1441,8 +1431,8 @@ __global__ void __launch_bounds__(32 * NW, LBM_WARP2_WARPS_PER_SM / NW)
         const float p0L = __shfl_up_sync(FULL, p0.v.y, 1), p0R = __shfl_down_sync(FULL, p0.v.x, 1);
         const float ppL = __shfl_up_sync(FULL, pp.v.y, 1), ppR = __shfl_down_sync(FULL, pp.v.x, 1);
         if (act_a) {
-            if (!(isfinite(mc.rho_d.v.x) && isfinite(mc.T_d.v.x)) ||
-                (act_b && !(isfinite(mc.rho_d.v.y) && isfinite(mc.T_d.v.y))))
+            if (!(lbm::finite(mc.rho_d.v.x) && lbm::finite(mc.T_d.v.x)) ||
+                (act_b && !(lbm::finite(mc.rho_d.v.y) && lbm::finite(mc.T_d.v.y))))
                 atomicOr(status, 1u);
             // the stencil for both nodes: left columns (xa - 1, xa), right (xb, xb + 1)
             auto grad = [&](const f2& cm, const f2& c0, const f2& cp, float mL, float mR, float zL, float zR, float pL,
@@ -1450,9 +1440,7 @@ __global__ void __launch_bounds__(32 * NW, LBM_WARP2_WARPS_PER_SM / NW)
                 const f2 lm(make_float2(mL, cm.v.x)), rmv(make_float2(cm.v.y, mR));
                 const f2 l0(make_float2(zL, c0.v.x)), r0v(make_float2(c0.v.y, zR));
                 const f2 lp(make_float2(pL, cp.v.x)), rpv(make_float2(cp.v.y, pR));
-                const f2 t(1.0f / 3.0f), d(1.0f / 12.0f);
-                gx = t * (r0v - l0) + d * ((rpv - lp) + (rmv - lm));
-                gy = t * (cp - cm) + d * ((rpv - rmv) + (lp - lm));
+                lbm::gradient3(lm, cm, rmv, l0, r0v, lp, cp, rpv, gx, gy);
             };
             f2 grx, gry, gpx, gpy;
             grad(rm, r0, rp, rmL, rmR, r0L, r0R, rpL, rpR, grx, gry);
@@ -1484,9 +1472,9 @@ __global__ void __launch_bounds__(32 * NW, LBM_WARP2_WARPS_PER_SM / NW)
                             const int dx = onW ? 1 : -1;
                             float r2, p2;
                             rho_p_at(P1, src, plane, pitch, x + 2 * dx, j, r2, p2);
-                            gxs = (float)dx * (-3.0f * v0 + 4.0f * (onW ? right : left) - (fld ? p2 : r2)) * 0.5f;
+                            gxs = (float)dx * (-3.0f * v0 + 4.0f * (onW ? right : left) - (fld ? p2 : r2)) * 1.5f;
                         } else {
-                            gxs = (right - left) * 0.5f;
+                            gxs = (right - left) * 1.5f;
                         }
                         const float vm = e ? cmf.v.y : cmf.v.x, vp = e ? cpf.v.y : cpf.v.x;
                         if (onS || onN) {
@@ -1494,9 +1482,9 @@ __global__ void __launch_bounds__(32 * NW, LBM_WARP2_WARPS_PER_SM / NW)
                             float r2, p2;
                             rho_p_at(P1, src, plane, pitch, x, j + 2 * dy, r2, p2);
                             const float v1 = onS ? vp : vm;
-                            gys = (float)dy * (-3.0f * v0 + 4.0f * v1 - (fld ? p2 : r2)) * 0.5f;
+                            gys = (float)dy * (-3.0f * v0 + 4.0f * v1 - (fld ? p2 : r2)) * 1.5f;
                         } else {
-                            gys = (vp - vm) * 0.5f;
+                            gys = (vp - vm) * 1.5f;
                         }
                         gr[2 * fld] = gxs;
                         gr[2 * fld + 1] = gys;
@@ -2135,9 +2123,9 @@ template <typename A, typename B>
 void convert_params(const Params<A>& a, Params<B>& b) {
 #define CP(f) b.f = (B)a.f
     CP(rho0); CP(T0); CP(E0); CP(Cv); CP(inv_Cv); CP(Rg); CP(eos_a); CP(eos_b); CP(p0); CP(rho0E0_p0);
-    CP(rho0Cp0); CP(mu0); CP(inv_T0); CP(visc_S); CP(lam_fac); CP(tj_fac); CP(e_fac); CP(alpha1);
-    CP(beta1); CP(alpha2); CP(beta2); CP(kk); CP(hh); CP(bb); CP(gamma1); CP(gamma2); CP(cR11);
-    CP(cR17); CP(cR18); CP(cR71); CP(cR77); CP(cR81); CP(cR88); CP(Fx); CP(Fy); CP(cs_b0); CP(dither);
+    CP(rho0Cp0); CP(mu0); CP(mu0S); CP(inv_T0); CP(visc_S); CP(lam_fac); CP(nu_e); CP(mu_j); CP(beta2);
+    CP(kk); CP(hh); CP(bb); CP(omk); CP(k2h); CP(gamma1); CP(gamma2); CP(k11); CP(k17); CP(k18);
+    CP(k71); CP(k77); CP(k81); CP(k88); CP(Fx); CP(Fy); CP(cs_b0); CP(dither);
 #undef CP
     b.eos = a.eos;
     b.visc = a.visc;
@@ -2863,29 +2851,34 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
     P.rho0E0_p0 = r0 * P.E0 + p0;
     P.rho0Cp0 = r0 * Cp;
     P.mu0 = r0 * (k.tau0 - 0.5) * cs2;
+    P.mu0S = P.mu0 * (1.0 + k.visc_p[0]);
     P.inv_T0 = 1.0 / T0;
     P.visc_S = k.visc_p[0];
     P.lam_fac = Cp / k.Pr;
     const double coef = 2.0 / 3.0 + k.gamma1 / 2.0 + k.gamma2 / 3.0;
     if (!(coef > 0)) return fail(LBM_EINVAL, "gamma1, gamma2 give a non-positive conductivity factor");
-    P.tj_fac = 1.0 / (coef * r0 * Cp);
-    P.e_fac = 3.0 * k.bulk_ratio / w;
-    P.alpha1 = -1.0;
-    P.beta1 = 1.0;
-    P.alpha2 = -(2.0 * P.alpha1 + w + 1.0) / (1.0 - w);
-    P.beta2 = -2.0 * P.beta1 / (1.0 - w);
+    P.mu_j = 2.0 * P.lam_fac / (coef * r0 * Cp);
+    const double e_fac = 3.0 * k.bulk_ratio / w;  // (1/s_e - 1/2) / nu
+    P.nu_e = 2.0 * e_fac;
+    // alpha1 = -1, beta1 = 1, so that alpha2 = -(2 alpha1 + w + 1) / (1 - w) = 1
+    P.beta2 = -2.0 / (1.0 - w);
     P.kk = 1.0 - w;
     P.hh = 6.0 * w * (1.0 - w) / (1.0 - 3.0 * w);
     P.bb = (1.0 - w) / (1.0 - 3.0 * w);
     P.gamma1 = k.gamma1;
     P.gamma2 = k.gamma2;
-    P.cR11 = -(9.0 - 15.0 * P.kk - 2.0 * P.hh) / (4.0 * w);
-    P.cR17 = -3.0 * (9.0 - 3.0 * P.kk + 2.0 * P.hh) / 4.0;
-    P.cR18 = 12.0 * (3.0 * P.kk + P.hh);
-    P.cR71 = -(3.0 - 4.0 * P.bb) / (4.0 * w);
-    P.cR77 = -3.0 * (3.0 + 4.0 * P.bb) / 4.0;
-    P.cR81 = P.bb / w;
-    P.cR88 = 6.0 * P.bb;
+    P.omk = 1.0 - P.kk;
+    P.k2h = 2.0 * P.kk + P.hh;
+    // entries of R without their velocity factors: s_e = 2 ic and s_p = 2 ia,
+    // s_p (2 - s_e) / (2 - s_p) = (2 e_fac / 3) ic, s_e (2 - s_p) / (2 - s_e) = (6 / e_fac) ia
+    const double q1 = 2.0 * e_fac / 3.0, q7 = 6.0 / e_fac;
+    P.k11 = -(9.0 - 15.0 * P.kk - 2.0 * P.hh) / (4.0 * w) * 2.0;
+    P.k17 = -3.0 * (9.0 - 3.0 * P.kk + 2.0 * P.hh) / 4.0 * q1;
+    P.k18 = 12.0 * (3.0 * P.kk + P.hh) * q1;
+    P.k71 = -(3.0 - 4.0 * P.bb) / (4.0 * w) * q7;
+    P.k77 = -3.0 * (3.0 + 4.0 * P.bb) / 4.0 * 2.0;
+    P.k81 = P.bb / w * q7;
+    P.k88 = 6.0 * P.bb * 2.0;
     P.Fx = k.force[0];
     P.Fy = k.force[1];
     P.cs_b0 = 1.0 - b * r0;
@@ -2913,8 +2906,8 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
         }
     }
 
-    const double eta0 = (p0 / cs2 - (2.0 + P.alpha1) * r0) / P.beta1;
-    const double mr[9] = {r0, 2.0 * P.alpha1 * r0 + 2.0 * P.beta1 * eta0, P.alpha2 * r0 + P.beta2 * eta0, 0, 0, 0, 0, 0, 0};
+    const double eta0 = p0 / cs2 - r0;  // (p0 / cs2 - (2 + alpha1) rho0) / beta1
+    const double mr[9] = {r0, -2.0 * r0 + 2.0 * eta0, r0 + P.beta2 * eta0, 0, 0, 0, 0, 0, 0};
     const double re = r0 * P.E0, rc = r0 * Cp * T0;
     const double nr[9] = {re, -4.0 * (re - rc) + k.gamma1 * rc, 4.0 * (re - rc) + k.gamma2 * rc, 0, 0, 0, 0, 0, 0};
     host_inverse_moments(mr, c->f_rest);
