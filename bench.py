@@ -112,7 +112,7 @@ def workload(name, precision):
 
 
 KERNEL_OF_PAIR = {0: "k_collide_stream", 1: "k_collide_pair", 2: "k_collide_pair", 3: "k_collide_stream",
-                  4: "k_collide_warp", 5: "k_collide_warp2"}
+                  4: "k_collide_warp", 5: "k_collide_warp2", 6: "k_collide_node"}
 KERNEL_SOURCES = ("lbm_gb300.cu", "lbm_node.cuh", "lbm_f2.cuh")
 
 

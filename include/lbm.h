@@ -202,9 +202,12 @@ lbm_status lbm_peak_rates(void* cuda_stream, double* out3);
  * and never synchronise with one another, bx = 30, 60 or 120 (1, 2 or 4
  * warps per CTA), any precision.  pair = 5 (FP32 storage only): warp
  * strips of 60 columns, two neighbouring nodes per lane in packed FP32,
- * bx = 60, 120 or 240.  pair = 0 and pair = 4 shapes of any width give
- * identical results; pairs 1-3 and 5 agree with them to FP32 rounding (their
- * arithmetic is contracted differently).  (bx, by, pair) = (0, 0, 0)
+ * bx = 60, 120 or 240.  pair = 6: node kernels, one launch that collides
+ * and pushes every node and one that rebuilds the wall nodes and writes every
+ * node's macros for the next step; bx = 128 nodes per CTA, by has no effect,
+ * any precision.  pair = 0, 4 and 6 shapes of any width give identical
+ * results; pairs 1-3 and 5 agree with them to FP32 rounding (pairs 1, 2 and
+ * 5 draw one random number per two nodes).  (bx, by, pair) = (0, 0, 0)
  * restores the default shape, which batches may then shorten.
  * Used by the autotuner. */
 lbm_status lbm_set_tile(lbm_ctx* ctx, int bx, int by, int pair);
@@ -219,7 +222,10 @@ lbm_status lbm_set_tile(lbm_ctx* ctx, int bx, int by, int pair);
  * up to 24 (FP32; 32 for pair = 1) or 8 (FP64) rows for members whose
  * shape was not set, shortened until the batch fills the GPU.  In either
  * case the runs that make up the last fill of the GPU in a launch are cut
- * into up to four runs of at least 6 rows, launched last. */
+ * into up to four runs of at least 6 rows, launched last.
+ * While a shape is the default, FP64 lattices, and FP32 lattices of few
+ * nodes (alone, or the FP32 members of a batch together), step through node
+ * kernels that give the bits of that shape, which stays what is reported. */
 lbm_status lbm_get_tile(const lbm_ctx* ctx, int* bx, int* by, int* pair);
 
 /* Steps taken since the last (re)initialisation. */

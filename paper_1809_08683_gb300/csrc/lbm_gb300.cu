@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <algorithm>
@@ -75,6 +76,8 @@ struct InstDesc {
     int nx, ny, pitch, px, py;
     int precision;
     unsigned int* status;
+    double* field;  // 5 nx ny doubles: node macros between k_prep and k_collide_node
+    int mc;         // model class (lbm::MODEL_*)
     WallDev wall[4];
     Params<double> pd;
     Params<float> pf;
@@ -89,6 +92,16 @@ struct Work {  // one CTA of the fused kernel
 struct BWork {  // one CTA of the wall pass
     int inst, k0, cnt, par;
 };
+
+struct NWork {  // one CTA of a node kernel (k_prep, k_collide_node)
+    int inst;
+    int n0, cnt;      // nodes n0 .. n0 + cnt - 1 in row-major order (k_collide_node2: pairs of nodes
+                      // of one row, (nx + 1) / 2 a row), or of the list of wall nodes
+    int kind;         // k_prep: kWallNodes or kInnerNodes
+    int par;
+    long long step0;  // the lattice's step count when this table was built
+};
+enum { kInnerNodes = 0, kWallNodes = 1 };
 
 template <typename R>
 __device__ __forceinline__ const Params<R>& dparams(const InstDesc* D);
@@ -619,11 +632,11 @@ __global__ void __launch_bounds__(BX, KEEP ? FusedTraits<R, BX>::MINB : FusedTra
                     R r2, p2;
                     rho_p_at<MC>(P, src, plane, pitch, x + 2 * dx, j, r2, p2);
                     const R r1 = s_rp[s0][c + dx].r, p1 = s_rp[s0][c + dx].p;
-                    grx = R(dx) * (R(-3) * r0 + R(4) * r1 - r2) * R(1.5);
-                    gpx = R(dx) * (R(-3) * p0 + R(4) * p1 - p2) * R(1.5);
+                    grx = lbm::onesided3(R(dx), r0, r1, r2);
+                    gpx = lbm::onesided3(R(dx), p0, p1, p2);
                 } else {
-                    grx = (s_rp[s0][c + 1].r - s_rp[s0][c - 1].r) * R(1.5);
-                    gpx = (s_rp[s0][c + 1].p - s_rp[s0][c - 1].p) * R(1.5);
+                    grx = lbm::central3(s_rp[s0][c - 1].r, s_rp[s0][c + 1].r);
+                    gpx = lbm::central3(s_rp[s0][c - 1].p, s_rp[s0][c + 1].p);
                 }
                 if (onS || onN) {
                     const int dy = onS ? 1 : -1;
@@ -631,11 +644,11 @@ __global__ void __launch_bounds__(BX, KEEP ? FusedTraits<R, BX>::MINB : FusedTra
                     rho_p_at<MC>(P, src, plane, pitch, x, j + 2 * dy, r2, p2);
                     const R r1 = onS ? s_rp[sp][c].r : s_rp[sm][c].r;
                     const R p1 = onS ? s_rp[sp][c].p : s_rp[sm][c].p;
-                    gry = R(dy) * (R(-3) * r0 + R(4) * r1 - r2) * R(1.5);
-                    gpy = R(dy) * (R(-3) * p0 + R(4) * p1 - p2) * R(1.5);
+                    gry = lbm::onesided3(R(dy), r0, r1, r2);
+                    gpy = lbm::onesided3(R(dy), p0, p1, p2);
                 } else {
-                    gry = (s_rp[sp][c].r - s_rp[sm][c].r) * R(1.5);
-                    gpy = (s_rp[sp][c].p - s_rp[sm][c].p) * R(1.5);
+                    gry = lbm::central3(s_rp[sm][c].r, s_rp[sp][c].r);
+                    gpy = lbm::central3(s_rp[sm][c].p, s_rp[sp][c].p);
                 }
             }
 
@@ -869,22 +882,22 @@ __global__ void __launch_bounds__(32 * NW, WarpTraits<R>::WARPS_PER_SM / NW)
                     R r2, p2;
                     rho_p_at<MC>(P, src, plane, pitch, x + 2 * dx, j, r2, p2);
                     const R r1 = onW ? r0r : r0l, p1 = onW ? p0r : p0l;
-                    grx = R(dx) * (R(-3) * r0 + R(4) * r1 - r2) * R(1.5);
-                    gpx = R(dx) * (R(-3) * p0 + R(4) * p1 - p2) * R(1.5);
+                    grx = lbm::onesided3(R(dx), r0, r1, r2);
+                    gpx = lbm::onesided3(R(dx), p0, p1, p2);
                 } else {
-                    grx = (r0r - r0l) * R(1.5);
-                    gpx = (p0r - p0l) * R(1.5);
+                    grx = lbm::central3(r0l, r0r);
+                    gpx = lbm::central3(p0l, p0r);
                 }
                 if (onS || onN) {
                     const int dy = onS ? 1 : -1;
                     R r2, p2;
                     rho_p_at<MC>(P, src, plane, pitch, x, j + 2 * dy, r2, p2);
                     const R r1 = onS ? rp : rm, p1 = onS ? pp : pm;
-                    gry = R(dy) * (R(-3) * r0 + R(4) * r1 - r2) * R(1.5);
-                    gpy = R(dy) * (R(-3) * p0 + R(4) * p1 - p2) * R(1.5);
+                    gry = lbm::onesided3(R(dy), r0, r1, r2);
+                    gpy = lbm::onesided3(R(dy), p0, p1, p2);
                 } else {
-                    gry = (rp - rm) * R(1.5);
-                    gpy = (pp - pm) * R(1.5);
+                    gry = lbm::central3(rm, rp);
+                    gpy = lbm::central3(pm, pp);
                 }
             }
 
@@ -945,7 +958,7 @@ __device__ void broadcast_params(const Params<float>& a, Params<f2>& b) {
 #define BP(f) b.f = f2(a.f)
     BP(rho0); BP(T0); BP(E0); BP(Cv); BP(inv_Cv); BP(Rg); BP(eos_a); BP(eos_b); BP(p0); BP(rho0E0_p0);
     BP(rho0Cp0); BP(mu0); BP(mu0S); BP(inv_T0); BP(visc_S); BP(lam_fac); BP(nu_e); BP(mu_j); BP(beta2);
-    BP(kk); BP(hh); BP(bb); BP(omk); BP(k2h); BP(gamma1); BP(gamma2); BP(k11); BP(k17); BP(k18);
+    BP(kk); BP(hh); BP(bb); BP(bbm2); BP(omk); BP(k2h); BP(gamma1); BP(gamma2); BP(k11); BP(k17); BP(k18);
     BP(k71); BP(k77); BP(k81); BP(k88); BP(Fx); BP(Fy); BP(cs_b0); BP(dither);
 #undef BP
     b.eos = a.eos;
@@ -1184,15 +1197,15 @@ __global__ void __launch_bounds__(BX / 2, (KEEP ? LBM_PAIR_WARPS_PER_SM : 12) * 
                         const float v0 = a[s0][c];
                         float gxs, gys;
                         if (onW || onE) {
-                            gxs = (float)dx * (-3.0f * v0 + 4.0f * a[s0][c + dx] - (fld ? px2 : rx2)) * 1.5f;
+                            gxs = lbm::onesided3((float)dx, v0, a[s0][c + dx], fld ? px2 : rx2);
                         } else {
-                            gxs = (a[s0][c + 1] - a[s0][c - 1]) * 1.5f;
+                            gxs = lbm::central3(a[s0][c - 1], a[s0][c + 1]);
                         }
                         if (onS || onN) {
                             const float v1 = onS ? a[sp][c] : a[sm][c];
-                            gys = (float)dy * (-3.0f * v0 + 4.0f * v1 - (fld ? py2 : ry2)) * 1.5f;
+                            gys = lbm::onesided3((float)dy, v0, v1, fld ? py2 : ry2);
                         } else {
-                            gys = (a[sp][c] - a[sm][c]) * 1.5f;
+                            gys = lbm::central3(a[sm][c], a[sp][c]);
                         }
                         gr[2 * fld] = gxs;
                         gr[2 * fld + 1] = gys;
@@ -1472,9 +1485,9 @@ __global__ void __launch_bounds__(32 * NW, LBM_WARP2_WARPS_PER_SM / NW)
                             const int dx = onW ? 1 : -1;
                             float r2, p2;
                             rho_p_at(P1, src, plane, pitch, x + 2 * dx, j, r2, p2);
-                            gxs = (float)dx * (-3.0f * v0 + 4.0f * (onW ? right : left) - (fld ? p2 : r2)) * 1.5f;
+                            gxs = lbm::onesided3((float)dx, v0, onW ? right : left, fld ? p2 : r2);
                         } else {
-                            gxs = (right - left) * 1.5f;
+                            gxs = lbm::central3(left, right);
                         }
                         const float vm = e ? cmf.v.y : cmf.v.x, vp = e ? cpf.v.y : cpf.v.x;
                         if (onS || onN) {
@@ -1482,9 +1495,9 @@ __global__ void __launch_bounds__(32 * NW, LBM_WARP2_WARPS_PER_SM / NW)
                             float r2, p2;
                             rho_p_at(P1, src, plane, pitch, x, j + 2 * dy, r2, p2);
                             const float v1 = onS ? vp : vm;
-                            gys = (float)dy * (-3.0f * v0 + 4.0f * v1 - (fld ? p2 : r2)) * 1.5f;
+                            gys = lbm::onesided3((float)dy, v0, v1, fld ? p2 : r2);
                         } else {
-                            gys = (vp - vm) * 1.5f;
+                            gys = lbm::central3(vm, vp);
                         }
                         gr[2 * fld] = gxs;
                         gr[2 * fld + 1] = gys;
@@ -1579,6 +1592,79 @@ __device__ void wall_node(const InstDesc* D, int k, WallNode& n) {
     }
 }
 
+// The wall node n's 18 populations rebuilt from its bounced sums, the wall
+// data and the extrapolated redefined non-equilibrium moments (Sec. 3).
+template <typename R>
+__device__ __forceinline__ void rebuilt_wall_node(const Params<R>& P, const R* __restrict__ buf, long long plane, int pitch,
+                                                  const WallNode& n, R* v) {
+    // the wall node's and x_f's populations, loaded together so that their
+    // latencies overlap (the pass is bound by them).  On a walled x side away
+    // from the corners the two nodes are neighbours in one row: when the
+    // pair starts on an even column it comes as one 8-byte (FP32) or
+    // 16-byte (FP64) load per population, which halves the load
+    // instructions and the DRAM sectors touched of a column of wall nodes.
+    R u[18];
+    const long long ib = (long long)n.y * pitch + n.x;
+    const int xl = n.dx > 0 ? n.x : n.x - 1;
+    if (n.dy == 0 && n.dx != 0 && (xl & 1) == 0) {
+        using V2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
+        const R* row = buf + (long long)n.y * pitch + xl;
+#pragma unroll
+        for (int q = 0; q < 18; ++q) {
+            const V2 pr = *reinterpret_cast<const V2*>(row + q * plane);
+            v[q] = n.dx > 0 ? pr.x : pr.y;
+            u[q] = n.dx > 0 ? pr.y : pr.x;
+        }
+    } else {
+        const R* a = buf + ib;
+        const R* b = buf + (long long)(n.y + n.dy) * pitch + (n.x + n.dx);
+#pragma unroll
+        for (int q = 0; q < 18; ++q) {
+            v[q] = a[q * plane];
+            u[q] = b[q * plane];
+        }
+    }
+    // density (and Neumann total energy) from the bounced-back populations
+    R rd, jx, jy, sg;
+    lbm::node_sums(v, v + 9, rd, jx, jy, sg);
+    const R ux = R(n.ux), uy = R(n.uy);
+    Mac<R> mb;
+    R rhoE_d;
+    if (n.thermal == 0) {
+        const R Td = R(n.T) - P.T0;
+        const R Ed = lbm::mad(P.Cv, Td, R(0.5) * lbm::mad(ux, ux, uy * uy));
+        rhoE_d = lbm::mad(rd, P.E0, (P.rho0 + rd) * Ed);
+    } else {
+        const R rho = P.rho0 + rd;
+        const R Fx = P.force_mode ? rho * P.Fx : P.Fx;
+        const R Fy = P.force_mode ? rho * P.Fy : P.Fy;
+        rhoE_d = lbm::mad(R(0.5), lbm::mad(ux, Fx, uy * Fy), sg);
+    }
+    lbm::wall_macros(P, rd, ux, uy, rhoE_d, mb);
+
+    // redefined non-equilibrium moments at x_f (and x_ff), extrapolated
+    R mt[9], nt[9];
+    {
+        Mac<R> m;
+        node_macros(P, u, m);
+        lbm::tilde_neq(P, m, u, u + 9, mt, nt);
+        if (n.order == 2) {
+            R mt2[9], nt2[9];
+            const R* c = buf + (long long)(n.y + 2 * n.dy) * pitch + (n.x + 2 * n.dx);
+#pragma unroll
+            for (int q = 0; q < 18; ++q) u[q] = c[q * plane];
+            node_macros(P, u, m);
+            lbm::tilde_neq(P, m, u, u + 9, mt2, nt2);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                mt[q] = lbm::mad(R(2), mt[q], -mt2[q]);
+                nt[q] = lbm::mad(R(2), nt[q], -nt2[q]);
+            }
+        }
+    }
+    lbm::rebuild(P, mb, mt, nt, v, v + 9);
+}
+
 // Resident CTAs per SM of the FP32 wall pass.  3 leaves 146 registers per
 // thread and no spills; 4 spilled 68 bytes per thread and took 0.1055 ms per
 // step of the 96-cavity batch against 0.098 ms (6 and 8 CTAs, with more
@@ -1601,73 +1687,286 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? LBM_BOUNDARY_MINB : 2) k
     load_params(&P, &dparams<R>(D));
     __syncthreads();
     if ((int)threadIdx.x >= w.cnt) return;
-    const int k = w.k0 + threadIdx.x;
-    const int pitch = D->pitch;
-    const long long plane = D->plane;
     R* __restrict__ buf = reinterpret_cast<R*>(D->buf[(w.par ^ step_par) ^ 1]);
     WallNode n;
-    wall_node(D, k, n);
+    wall_node(D, w.k0 + threadIdx.x, n);
+    R v[18];
+    rebuilt_wall_node(P, buf, D->plane, D->pitch, n, v);
+    store18<R>(buf, D->plane, (long long)n.y * D->pitch + n.x, v);
+}
 
-    // the wall node's and x_f's populations, loaded together so that their
-    // latencies overlap (the pass is bound by them).  On a walled x side away
-    // from the corners the two nodes are neighbours in one row: when the
-    // pair starts on an even column it comes as one 8-byte (FP32) or
-    // 16-byte (FP64) load per population, which halves the load
-    // instructions and the DRAM sectors touched of a column of wall nodes.
-    R v[18], u[18];
-    const long long ib = (long long)n.y * pitch + n.x;
-    const int xl = n.dx > 0 ? n.x : n.x - 1;
-    if (n.dy == 0 && n.dx != 0 && (xl & 1) == 0) {
-        using V2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
-        const R* row = buf + (long long)n.y * pitch + xl;
-#pragma unroll
-        for (int q = 0; q < 18; ++q) {
-            const V2 pr = __ldg(reinterpret_cast<const V2*>(row + q * plane));
-            v[q] = n.dx > 0 ? pr.x : pr.y;
-            u[q] = n.dx > 0 ? pr.y : pr.x;
+// ------------------------------------------------------------------------
+// one node per thread: k_prep and k_collide_node
+// ------------------------------------------------------------------------
+
+// A step of a lattice whose DFs stay in L2, or whose arithmetic is FP64, as
+// two launches over all its nodes in row-major order, 128 per CTA:
+//   k_collide_node   collides and pushes every node; rho' and p' of its
+//                    neighbours come from the lattice's field array;
+//   k_prep           rebuilds the wall nodes of the buffer pushed into (what
+//                    k_boundary does for the strips) and writes every node's
+//                    macros to the field array for the next step.
+// The strips compute the macros of their halo rows and columns again (2 of 8
+// rows, and one warp instruction per halo column whatever its lanes) and
+// leave lanes idle on a ragged edge.  FP64 is bound by its instruction count
+// (one per 76 cycles and scheduler), small FP32 lattices by latency and by
+// the number of warps in flight; neither is bound by the extra traffic (the
+// DFs are read twice, and 16 B (FP32) or 80 B (FP64) of macros written and
+// read per node).  The arithmetic is that of the strips and so are the bits.
+// Time of a pass against the strips: 64 lattices of sides 64-128, 20 FP64
+// steps 10.9 -> 7.3 ms; 512^2 FP64, 20 steps 5.61 -> 4.41 ms; 64 lattices,
+// 50 FP32 steps 3.53 -> 2.82 ms; 512^2 FP32, 100 steps 2.73 -> 2.47 ms.
+
+// The field array as seen by the kernels: rho', p' pairs, and (FP64, where
+// forming them again costs more than reading them) ux, uy and T'.
+template <typename R>
+struct Field {
+    RhoP<R>* rp;
+    R *ux, *uy, *T;
+    __device__ __forceinline__ Field(double* base, long long nn)
+        : rp(reinterpret_cast<RhoP<R>*>(base)), ux(reinterpret_cast<R*>(rp + nn)), uy(ux + nn), T(uy + nn) {}
+};
+constexpr int kNodeThreads = 128;
+
+// wall_mode 0: macros of every node of the current buffer, as it stands
+// (first launch of a stepping call).  wall_mode 1: after a step, on the
+// buffer that it pushed into.
+template <typename R>
+__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 4 : 2)
+    k_prep(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int step_par, int wall_mode,
+           long long* __restrict__ counter) {
+    __shared__ Params<R> P;
+    if (counter && blockIdx.x == 0 && threadIdx.x == 0) *counter += 1;
+    const NWork w = work[blockIdx.x];
+    const InstDesc* D = descs[w.inst];
+    load_params(&P, &dparams<R>(D));
+    __syncthreads();
+    if ((int)threadIdx.x >= w.cnt) return;
+    const int nx = D->nx, ny = D->ny, pitch = D->pitch;
+    const long long plane = D->plane;
+    R* __restrict__ buf = reinterpret_cast<R*>(D->buf[w.par ^ step_par ^ wall_mode]);
+    const int k = w.n0 + threadIdx.x;
+    int x, y;
+    R v[18];
+    if (w.kind == kWallNodes) {
+        WallNode n;
+        wall_node(D, k, n);
+        x = n.x;
+        y = n.y;
+        if (wall_mode) {
+            rebuilt_wall_node(P, buf, plane, pitch, n, v);
+            store18<R>(buf, plane, (long long)y * pitch + x, v);
         }
     } else {
-        load18<R>(buf, plane, ib, v);
-        load18<R>(buf, plane, (long long)(n.y + n.dy) * pitch + (n.x + n.dx), u);
+        y = k / nx;
+        x = k - y * nx;
+        if ((!D->px && (x == 0 || x == nx - 1)) || (!D->py && (y == 0 || y == ny - 1))) return;
     }
-    // density (and Neumann total energy) from the bounced-back populations
-    R rd, jx, jy, sg;
-    lbm::node_sums(v, v + 9, rd, jx, jy, sg);
-    const R ux = R(n.ux), uy = R(n.uy);
-    Mac<R> mb;
-    R rhoE_d;
-    if (n.thermal == 0) {
-        const R Td = R(n.T) - P.T0;
-        const R Ed = P.Cv * Td + R(0.5) * (ux * ux + uy * uy);
-        rhoE_d = rd * P.E0 + (P.rho0 + rd) * Ed;
-    } else {
-        const R rho = P.rho0 + rd;
-        const R Fx = P.force_mode ? rho * P.Fx : P.Fx;
-        const R Fy = P.force_mode ? rho * P.Fy : P.Fy;
-        rhoE_d = sg + R(0.5) * (ux * Fx + uy * Fy);
-    }
-    lbm::wall_macros(P, rd, ux, uy, rhoE_d, mb);
-
-    // redefined non-equilibrium moments at x_f (and x_ff), extrapolated
-    R mt[9], nt[9];
-    {
-        Mac<R> m;
-        node_macros(P, u, m);
-        lbm::tilde_neq(P, m, u, u + 9, mt, nt);
-        if (n.order == 2) {
-            R mt2[9], nt2[9];
-            load18<R>(buf, plane, (long long)(n.y + 2 * n.dy) * pitch + (n.x + 2 * n.dx), u);
-            node_macros(P, u, m);
-            lbm::tilde_neq(P, m, u, u + 9, mt2, nt2);
+    if (!(w.kind == kWallNodes && wall_mode)) {
+        const R* a = buf + (long long)y * pitch + x;
 #pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                mt[q] = R(2) * mt[q] - mt2[q];
-                nt[q] = R(2) * nt[q] - nt2[q];
+        for (int q = 0; q < 18; ++q) v[q] = a[q * plane];
+    }
+    Mac<R> m;
+    node_macros(P, v, m);
+    const Field<R> F(D->field, (long long)nx * ny);
+    const int t = y * nx + x;
+    F.rp[t] = RhoP<R>{m.rho_d, m.p_d};
+    if (sizeof(R) == 8) {
+        F.ux[t] = m.ux;
+        F.uy[t] = m.uy;
+        F.T[t] = m.T_d;
+    }
+}
+
+template <typename R, int MC>
+__device__ __forceinline__ void collide_node(const NWork& w, const InstDesc* D, const Params<R>& P, int step_par, uint32_t step_hash) {
+    const int nx = D->nx, ny = D->ny, pitch = D->pitch, px = D->px, py = D->py;
+    const long long plane = D->plane;
+    const int b = w.par ^ step_par;
+    const R* __restrict__ src = reinterpret_cast<const R*>(D->buf[b]);
+    R* __restrict__ dst = reinterpret_cast<R*>(D->buf[b ^ 1]);
+    const int t = w.n0 + threadIdx.x;
+    const int y = t / nx, x = t - y * nx;
+    R v[18];
+    load18<R>(src, plane, (long long)y * pitch + x, v);
+
+    // three times the gradients of rho and p; offsets of the neighbouring
+    // columns and rows with the wrap of a periodic side
+    const Field<R> F(D->field, (long long)nx * ny);
+    const RhoP<R>* __restrict__ rp = F.rp + t;
+    const int xl = x > 0 ? -1 : nx - 1, xr = x < nx - 1 ? 1 : 1 - nx;
+    const int yd = y > 0 ? -nx : (ny - 1) * nx, yu = y < ny - 1 ? nx : (1 - ny) * nx;
+    const RhoP<R> c = rp[0], zl = rp[xl], zr = rp[xr], mc_ = rp[yd], pc = rp[yu];
+    const bool onW = !px && x == 0, onE = !px && x == nx - 1, onS = !py && y == 0, onN = !py && y == ny - 1;
+    R grx, gry, gpx, gpy;
+    if (!(onW || onE || onS || onN)) {
+        const RhoP<R> ml = rp[yd + xl], mr = rp[yd + xr], pl = rp[yu + xl], pr = rp[yu + xr];
+        lbm::gradient3(ml.r, mc_.r, mr.r, zl.r, zr.r, pl.r, pc.r, pr.r, grx, gry);
+        lbm::gradient3(ml.p, mc_.p, mr.p, zl.p, zr.p, pl.p, pc.p, pr.p, gpx, gpy);
+    } else {
+        // wall node: one-sided second order along the inward normal,
+        // central along the wall (three times each, as gradient3)
+        if (onW || onE) {
+            const int dx = onW ? 1 : -1;
+            const RhoP<R> n1 = rp[dx], n2 = rp[2 * dx];
+            grx = lbm::onesided3(R(dx), c.r, n1.r, n2.r);
+            gpx = lbm::onesided3(R(dx), c.p, n1.p, n2.p);
+        } else {
+            grx = lbm::central3(zl.r, zr.r);
+            gpx = lbm::central3(zl.p, zr.p);
+        }
+        if (onS || onN) {
+            const int dy = onS ? 1 : -1;
+            const RhoP<R> n1 = rp[dy * nx], n2 = rp[2 * dy * nx];
+            gry = lbm::onesided3(R(dy), c.r, n1.r, n2.r);
+            gpy = lbm::onesided3(R(dy), c.p, n1.p, n2.p);
+        } else {
+            gry = lbm::central3(mc_.r, pc.r);
+            gpy = lbm::central3(mc_.p, pc.p);
+        }
+    }
+
+    Mac<R> m;
+    if (sizeof(R) == 8) {
+        MacC<R> mk;
+        mk.rho_d = c.r;
+        mk.ir = lbm::recip(P.rho0 + c.r);
+        mk.ux = F.ux[t];
+        mk.uy = F.uy[t];
+        mk.T_d = F.T[t];
+        mk.p_d = c.p;
+        R rd, jx, jy, sg;
+        lbm::node_sums(v, v + 9, rd, jx, jy, sg);  // only sg is used
+        mk.rhoE_d = sg;
+        lbm::expand<MC>(P, mk, m);
+        m.rhoE_d = lbm::mad(R(0.5), m.qe, sg);
+        m.rhoH = P.rho0E0_p0 + m.rhoE_d + m.p_d;
+    } else {
+        node_macros<MC>(P, v, m);
+    }
+    if (!(lbm::finite(m.rho_d) && lbm::finite(m.T_d))) atomicOr(D->status, 1u);
+    AddDither add(mix32(step_hash ^ ((uint32_t)y * 0x85ebca77u + (uint32_t)x * 0xc2b2ae3du)), (float)P.dither);
+    lbm::collide<MC>(P, m, v, v + 9, grx, gry, gpx, gpy, add);
+    push_node(dst, v, x, y, nx, ny, pitch, plane, px, py);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 4 : 2)
+    k_collide_node(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int step_par,
+                   const long long* __restrict__ counter) {
+    __shared__ Params<R> P;
+    const NWork w = work[blockIdx.x];
+    const InstDesc* D = descs[w.inst];
+    load_params(&P, &dparams<R>(D));
+    const uint32_t step_hash = mix32((uint32_t)(w.step0 + *counter) * 0x9e3779b1u + 0x632be5abu);
+    __syncthreads();
+    if ((int)threadIdx.x >= w.cnt) return;
+    if (D->mc == lbm::MODEL_CAVITY) collide_node<R, lbm::MODEL_CAVITY>(w, D, P, step_par, step_hash);
+    else collide_node<R, lbm::MODEL_ANY>(w, D, P, step_par, step_hash);
+}
+
+// k_collide_node for two neighbouring nodes per thread in packed FP32: the
+// arithmetic and the rounding draws of k_collide_pair, for the lattices whose
+// strips those are.
+template <int MC>
+__device__ __forceinline__ void collide_node2(const NWork& w, const InstDesc* D, const Params<f2>& P, float dscale, int step_par,
+                                              uint32_t step_hash) {
+    const int nx = D->nx, ny = D->ny, pitch = D->pitch, px = D->px, py = D->py;
+    const long long plane = D->plane;
+    const int b = w.par ^ step_par;
+    const float* __restrict__ src = reinterpret_cast<const float*>(D->buf[b]);
+    float* __restrict__ dst = reinterpret_cast<float*>(D->buf[b ^ 1]);
+    const int per_row = (nx + 1) >> 1, t2 = w.n0 + threadIdx.x;
+    const int y = t2 / per_row, xa = 2 * (t2 - y * per_row), xb = xa + 1;
+    const bool act_b = xb < nx;
+    f2 v[18];
+    const float* sp = src + (long long)y * pitch + xa;
+#pragma unroll
+    for (int q = 0; q < 18; ++q) v[q] = f2(__ldg(reinterpret_cast<const float2*>(sp + q * plane)));
+
+    // rows y - 1 (m), y (z), y + 1 (p) of the field at columns xa - 1, xa,
+    // xa + 1, xa + 2, wrapped across a periodic side; without column xa + 1,
+    // the right neighbour of xa takes its place
+    const Field<float> F(D->field, (long long)nx * ny);
+    const RhoP<float>* __restrict__ rp = F.rp + (long long)y * nx;
+    const int cl = xa > 0 ? xa - 1 : nx - 1, cb = act_b ? xb : (px ? 0 : xa), cr = xb < nx - 1 ? xb + 1 : (xb - nx + 1) % nx;
+    const int ym = y > 0 ? -nx : (ny - 1) * nx, yp = y < ny - 1 ? nx : (1 - ny) * nx;
+    struct Row {
+        RhoP<float> l, a, b, r;
+    };
+    auto row = [&](int off) { return Row{rp[off + cl], rp[off + xa], rp[off + cb], rp[off + cr]}; };
+    const Row m = row(ym), z = row(0), p = row(yp);
+    f2 grx, gry, gpx, gpy;
+    auto pack = [](float u, float v2) { return f2(make_float2(u, v2)); };
+    lbm::gradient3(pack(m.l.r, m.a.r), pack(m.a.r, m.b.r), pack(m.b.r, m.r.r), pack(z.l.r, z.a.r), pack(z.b.r, z.r.r),
+                   pack(p.l.r, p.a.r), pack(p.a.r, p.b.r), pack(p.b.r, p.r.r), grx, gry);
+    lbm::gradient3(pack(m.l.p, m.a.p), pack(m.a.p, m.b.p), pack(m.b.p, m.r.p), pack(z.l.p, z.a.p), pack(z.b.p, z.r.p),
+                   pack(p.l.p, p.a.p), pack(p.a.p, p.b.p), pack(p.b.p, p.r.p), gpx, gpy);
+    const bool onS = !py && y == 0, onN = !py && y == ny - 1;
+    if (onS || onN || (!px && (xa == 0 || xb >= nx - 1))) {
+        // wall nodes: one-sided second order along the inward normal, central
+        // along the wall (three times each, as gradient3)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int x = e ? xb : xa;
+            const bool onW = !px && x == 0, onE = !px && x == nx - 1;
+            if ((e && !act_b) || !(onS || onN || onW || onE)) continue;
+            const RhoP<float> c = e ? z.b : z.a, lo = e ? m.b : m.a, hi = e ? p.b : p.a;
+            float gr[4];
+            if (onW || onE) {
+                const int dx = onW ? 1 : -1;
+                const RhoP<float> n1 = rp[x + dx], n2 = rp[x + 2 * dx];
+                gr[0] = lbm::onesided3((float)dx, c.r, n1.r, n2.r);
+                gr[1] = lbm::onesided3((float)dx, c.p, n1.p, n2.p);
+            } else {
+                const RhoP<float> l = e ? z.a : z.l, r = e ? z.r : z.b;
+                gr[0] = lbm::central3(l.r, r.r);
+                gr[1] = lbm::central3(l.p, r.p);
             }
+            if (onS || onN) {
+                const int dy = onS ? 1 : -1;
+                const RhoP<float> n1 = rp[x + dy * nx], n2 = rp[x + 2 * dy * nx];
+                gr[2] = lbm::onesided3((float)dy, c.r, n1.r, n2.r);
+                gr[3] = lbm::onesided3((float)dy, c.p, n1.p, n2.p);
+            } else {
+                gr[2] = lbm::central3(lo.r, hi.r);
+                gr[3] = lbm::central3(lo.p, hi.p);
+            }
+            if (e) { grx.v.y = gr[0]; gpx.v.y = gr[1]; gry.v.y = gr[2]; gpy.v.y = gr[3]; }
+            else { grx.v.x = gr[0]; gpx.v.x = gr[1]; gry.v.x = gr[2]; gpy.v.x = gr[3]; }
         }
     }
-    lbm::rebuild(P, mb, mt, nt, v, v + 9);
-    store18<R>(buf, plane, ib, v);
+
+    f2 rd, jx, jy, sg;
+    lbm::node_sums(v, v + 9, rd, jx, jy, sg);
+    Mac<f2> mf;
+    lbm::macros<MC>(P, rd, jx, jy, sg, mf);
+    if (!(lbm::finite(mf.rho_d.v.x) && lbm::finite(mf.T_d.v.x)) ||
+        (act_b && !(lbm::finite(mf.rho_d.v.y) && lbm::finite(mf.T_d.v.y))))
+        atomicOr(D->status, 1u);
+    AddDither2 add(mix32(step_hash ^ ((uint32_t)y * 0x85ebca77u + (uint32_t)xa * 0xc2b2ae3du)), dscale);
+    lbm::collide<MC>(P, mf, v, v + 9, grx, gry, gpx, gpy, add);
+    push_pair(dst, v, xa, act_b, y, nx, ny, pitch, plane, px, py);
+}
+
+__global__ void __launch_bounds__(kNodeThreads, 3)
+    k_collide_node2(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int step_par,
+                    const long long* __restrict__ counter) {
+    __shared__ Params<f2> P;
+    const NWork w = work[blockIdx.x];
+    const InstDesc* D = descs[w.inst];
+    // Params<f2> holds each number of Params<float> twice, then the same four integers
+    constexpr int nf = offsetof(Params<float>, eos) / sizeof(float);
+    static_assert(offsetof(Params<f2>, eos) == nf * sizeof(f2), "Params is numbers, then integers");
+    const float* pf = reinterpret_cast<const float*>(&D->pf);
+    for (int i = threadIdx.x; i < nf; i += kNodeThreads) reinterpret_cast<float2*>(&P)[i] = make_float2(pf[i], pf[i]);
+    if (threadIdx.x < 4) reinterpret_cast<int*>(&P.eos)[threadIdx.x] = reinterpret_cast<const int*>(&D->pf.eos)[threadIdx.x];
+    const uint32_t step_hash = mix32((uint32_t)(w.step0 + *counter) * 0x9e3779b1u + 0x632be5abu);
+    __syncthreads();
+    if ((int)threadIdx.x >= w.cnt) return;
+    if (D->mc == lbm::MODEL_CAVITY) collide_node2<lbm::MODEL_CAVITY>(w, D, P, D->pf.dither, step_par, step_hash);
+    else collide_node2<lbm::MODEL_ANY>(w, D, P, D->pf.dither, step_par, step_hash);
 }
 
 // ------------------------------------------------------------------------
@@ -1701,8 +2000,8 @@ __global__ void k_init_macros(const InstDesc* D, int b, const double* __restrict
         const int y = (int)(t / D->nx), x = (int)(t % D->nx);
         const double rd = rho[t] - Pd.rho0;
         const double u = ux[t], vv = uy[t];
-        const double Ed = Pd.Cv * (T[t] - Pd.T0) + 0.5 * (u * u + vv * vv);
-        const double rhoE_d = rd * Pd.E0 + rho[t] * Ed;
+        const double Ed = lbm::mad(Pd.Cv, T[t] - Pd.T0, 0.5 * lbm::mad(u, u, vv * vv));
+        const double rhoE_d = lbm::mad(rd, Pd.E0, rho[t] * Ed);
         Mac<R> m;
         lbm::wall_macros(P, R(rd), R(u), R(vv), R(rhoE_d), m);
         R v[18];
@@ -1821,14 +2120,14 @@ __device__ __forceinline__ void diag_partials(const InstDesc* D, int b, double* 
         acc[0] += m.rho_d;
         acc[1] += m.rhoE_d;
         acc[2] += wx * wy * p / (D->pd.p0 * Lx * Ly);
-        const double u2 = m.ux * m.ux + m.uy * m.uy;
+        const double u2 = lbm::mad(m.ux, m.ux, m.uy * m.uy);
         if (have_snapshot) {
             const double dux = m.ux - snap[t], duy = m.uy - snap[nn + t], dT = m.T - snap[2 * nn + t];
-            acc[3] += dux * dux + duy * duy;
-            acc[5] += dT * dT;
+            acc[3] += lbm::mad(dux, dux, duy * duy);
+            acc[5] = lbm::mad(dT, dT, acc[5]);
         }
         acc[4] += u2;
-        acc[6] += m.T_d * m.T_d;
+        acc[6] = lbm::mad(m.T_d, m.T_d, acc[6]);
         acc[8] = fmax(acc[8], sqrt(u2));
         acc[9] += m.T;
         if (take_snapshot) {
@@ -2124,7 +2423,7 @@ void convert_params(const Params<A>& a, Params<B>& b) {
 #define CP(f) b.f = (B)a.f
     CP(rho0); CP(T0); CP(E0); CP(Cv); CP(inv_Cv); CP(Rg); CP(eos_a); CP(eos_b); CP(p0); CP(rho0E0_p0);
     CP(rho0Cp0); CP(mu0); CP(mu0S); CP(inv_T0); CP(visc_S); CP(lam_fac); CP(nu_e); CP(mu_j); CP(beta2);
-    CP(kk); CP(hh); CP(bb); CP(omk); CP(k2h); CP(gamma1); CP(gamma2); CP(k11); CP(k17); CP(k18);
+    CP(kk); CP(hh); CP(bb); CP(bbm2); CP(omk); CP(k2h); CP(gamma1); CP(gamma2); CP(k11); CP(k17); CP(k18);
     CP(k71); CP(k77); CP(k81); CP(k88); CP(Fx); CP(Fy); CP(cs_b0); CP(dither);
 #undef CP
     b.eos = a.eos;
@@ -2162,6 +2461,8 @@ struct lbm_ctx {
     int device = 0;         // device current at lbm_create, which holds the workspace
     BWork* d_bwork = nullptr;
     int n_bwork = 0;
+    NWork* d_nwork = nullptr;  // node kernels: n_node items of k_collide_node, then n_prep of k_prep
+    int n_node = 0, n_prep = 0;
     long steps = 0;
     bool eos_set = false, have_snap = false;
     lbm_status sticky = LBM_OK;
@@ -2169,6 +2470,7 @@ struct lbm_ctx {
     double f_rest[9] = {0}, g_rest[9] = {0};
     std::vector<Work> h_work;
     std::vector<BWork> h_bwork;
+    std::vector<NWork> h_nwork;
 };
 
 // Fused-kernel variants: strips of 32, 64, 128 columns, one node per thread
@@ -2179,13 +2481,21 @@ struct lbm_ctx {
 // pair = 3); one autonomous warp per 30 columns, 1, 2 or 4 warps per CTA
 // (indices 12-14, pair = 4); one autonomous warp per 60 columns, two nodes
 // per lane in packed FP32 (indices 15-17, pair = 5).  Variants 3-11 and
-// 15-17 need FP32 storage.
-constexpr int kVariants = 18;
+// 15-17 need FP32 storage.  Variant 18 (pair = 6) is the node kernels, whose
+// work items are NWork, not Work.
+constexpr int kVariants = 19;
 constexpr int kModels = 2;  // model classes: lbm::MODEL_ANY, lbm::MODEL_CAVITY
 // Lattices below this many nodes keep the generic instance even with the
 // cavity model: they are latency-bound, and batches of them (the serving
 // mix) then stay one launch per shape.
 constexpr long long kModelMinNodes = 32768;
+// Most FP32 nodes that default shapes step through the node kernels: two
+// lattices of 72 B per node and the 8 B of macros stay below twice the 129 MB
+// of L2, beyond which the node kernels' second read of the DFs comes from HBM.
+#ifndef LBM_NODE_MAX_FP32
+#define LBM_NODE_MAX_FP32 1500000
+#endif
+constexpr long long kNodeMaxFp32 = LBM_NODE_MAX_FP32;
 
 // The launches of one time step over a set of members: launch groups
 // [precision][variant][model class] as ranges of the batch's work table,
@@ -2194,6 +2504,10 @@ constexpr long long kModelMinNodes = 32768;
 struct LaunchSet {
     int w_off[2][kVariants][kModels] = {}, w_cnt[2][kVariants][kModels] = {};
     int b_off[2] = {0, 0}, b_cnt[2] = {0, 0};
+    // node kernels: [kind] ranges of the batch's table of node work for the
+    // collision, [precision] ranges for k_prep
+    int n_off[3] = {0, 0, 0}, n_cnt[3] = {0, 0, 0};
+    int p_off[2] = {0, 0}, p_cnt[2] = {0, 0};
     long long* counter = nullptr;
 };
 
@@ -2204,6 +2518,7 @@ struct lbm_batch {
     InstDesc** d_descs = nullptr;
     Work* d_work = nullptr;
     BWork* d_bwork = nullptr;
+    NWork* d_nwork = nullptr;
     LaunchSet set;                   // every member's launches of one time step
     long steps = 0;
     int graph_steps = 0;
@@ -2290,6 +2605,38 @@ void ensure_tick(std::vector<BWork>& v, int inst, int par) {
         v.push_back(b);
     }
 }
+
+// Work items of the node kernels for one lattice: every node for
+// k_collide_node; the wall nodes, whose work is longest, and then the rows
+// that hold other nodes for k_prep.
+void add_node_work(const lbm_config& c, int inst, int par, bool pairs, long long step0, std::vector<NWork>& v) {
+    const long long nn = (long long)(pairs ? (c.nx + 1) / 2 : c.nx) * c.ny;
+    for (long long n0 = 0; n0 < nn; n0 += kNodeThreads)
+        v.push_back(NWork{inst, (int)n0, (int)std::min<long long>(kNodeThreads, nn - n0), kInnerNodes, par, step0});
+}
+void add_prep_wall(const lbm_config& c, int inst, int par, std::vector<NWork>& v) {
+    const int n = wall_count(c.nx, c.ny, c.wall[LBM_WALL_W].periodic != 0, c.wall[LBM_WALL_S].periodic != 0);
+    for (int n0 = 0; n0 < n; n0 += kNodeThreads)
+        v.push_back(NWork{inst, n0, std::min(kNodeThreads, n - n0), kWallNodes, par, 0});
+}
+void add_prep_inner(const lbm_config& c, int inst, int par, std::vector<NWork>& v) {
+    const int edge = c.wall[LBM_WALL_S].periodic ? 0 : 1;
+    const long long hi = (long long)c.nx * (c.ny - edge);
+    for (long long n0 = (long long)c.nx * edge; n0 < hi; n0 += kNodeThreads)
+        v.push_back(NWork{inst, (int)n0, (int)std::min<long long>(kNodeThreads, hi - n0), kInnerNodes, par, 0});
+}
+
+// Whether a lattice steps through the node kernels: always when lbm_set_tile
+// chose them; with a default shape, FP64 lattices always, and FP32 lattices
+// while the nodes stepped together (`nodes`: one lattice, or a batch's FP32
+// members) are few enough.  See kNodeMaxFp32.
+bool node_kernels(const lbm_ctx* c, long long nodes) {
+    if (c->tile_set) return c->pair == 6;
+    return c->cfg.precision == LBM_FP64 || nodes <= kNodeMaxFp32;
+}
+// Which of them: 0 FP64, 1 FP32, 2 FP32 in pairs (lattices whose strips are paired).
+enum { kNode64 = 0, kNode32 = 1, kNodePair = 2, kNodeKinds = 3 };
+int node_kind(const lbm_ctx* c) { return c->cfg.precision == LBM_FP64 ? kNode64 : c->pair == 1 ? kNodePair : kNode32; }
 
 // Default launch shape.  Lattices up to 160 columns wide take warp strips
 // of 30 columns (pair 4, same bits as pair 0): they waste fewer lanes there
@@ -2386,6 +2733,20 @@ bool is_fp32(const lbm_ctx* c);
 
 lbm_status upload_work(lbm_ctx* c) {
     if (c->d_work) { cudaFree(c->d_work); c->d_work = nullptr; }
+    if (c->d_nwork) { cudaFree(c->d_nwork); c->d_nwork = nullptr; }
+    c->n_node = c->n_prep = 0;
+    if (node_kernels(c, (long long)c->cfg.nx * c->cfg.ny)) {
+        std::vector<NWork>& v = c->h_nwork;
+        v.clear();
+        add_node_work(c->cfg, 0, 0, node_kind(c) == kNodePair, 0, v);
+        c->n_node = (int)v.size();
+        add_prep_wall(c->cfg, 0, 0, v);
+        add_prep_inner(c->cfg, 0, 0, v);
+        c->n_prep = (int)v.size() - c->n_node;
+        CUDA_TRY(cudaMalloc(&c->d_nwork, v.size() * sizeof(NWork)));
+        CUDA_TRY(cudaMemcpyAsync(c->d_nwork, v.data(), v.size() * sizeof(NWork), cudaMemcpyHostToDevice, c->stream));
+        return LBM_OK;
+    }
     c->h_work = make_work(c->cfg, 0, c->bx, c->by, 0, 0);
     split_tail(c->h_work, resident_ctas(variant_index(c->bx, c->pair), is_fp32(c)));
     c->n_work = (int)c->h_work.size();
@@ -2575,8 +2936,8 @@ void launch_pair_bx(const Work* work, int n, InstDesc* const* descs, int par, co
 }
 
 static const int kVariantWidth[kVariants] = {32, 64, 128, 64, 128, 256, 64, 128, 256, 32, 64, 128, 30, 60, 120,
-                                            60, 120, 240};
-static const int kVariantPair[kVariants] = {0, 0, 0, 1, 1, 1, 2, 2, 2, 3, 3, 3, 4, 4, 4, 5, 5, 5};
+                                            60, 120, 240, kNodeThreads};
+static const int kVariantPair[kVariants] = {0, 0, 0, 1, 1, 1, 2, 2, 2, 3, 3, 3, 4, 4, 4, 5, 5, 5, 6};
 
 int variant_index(int bx, int pair) {
     for (int v = 0; v < kVariants; ++v)
@@ -2644,6 +3005,19 @@ void launch_boundary(const BWork* work, int n, InstDesc* const* descs, int par, 
                      cudaStream_t s) {
     if (n <= 0) return;
     k_boundary<R><<<n, 128, 0, s>>>(work, descs, par, counter);
+}
+
+void launch_node(int kind, const NWork* work, int n, InstDesc* const* descs, int par, const long long* counter, cudaStream_t s) {
+    if (n <= 0) return;
+    if (kind == kNodePair) k_collide_node2<<<n, kNodeThreads, 0, s>>>(work, descs, par, counter);
+    else if (kind == kNode32) k_collide_node<float><<<n, kNodeThreads, 0, s>>>(work, descs, par, counter);
+    else k_collide_node<double><<<n, kNodeThreads, 0, s>>>(work, descs, par, counter);
+}
+void launch_prep(bool fp32, const NWork* work, int n, InstDesc* const* descs, int par, int wall_mode, long long* counter,
+                 cudaStream_t s) {
+    if (n <= 0) return;
+    if (fp32) k_prep<float><<<n, kNodeThreads, 0, s>>>(work, descs, par, wall_mode, counter);
+    else k_prep<double><<<n, kNodeThreads, 0, s>>>(work, descs, par, wall_mode, counter);
 }
 
 int grid_for(long long nn) {
@@ -2752,6 +3126,7 @@ lbm_status lbm_create(const lbm_config* cfg, void* workspace, size_t workspace_b
     h.py = cfg->wall[LBM_WALL_S].periodic != 0;
     h.precision = cfg->precision;
     h.status = c->d_status;
+    h.field = c->d_stage;
     for (int s = 0; s < 4; ++s) {
         h.wall[s].u[0] = cfg->wall[s].u[0];
         h.wall[s].u[1] = cfg->wall[s].u[1];
@@ -2791,6 +3166,7 @@ lbm_status lbm_destroy(lbm_ctx* c) {
     else cudaDeviceSynchronize();
     if (c->d_work) cudaFree(c->d_work);
     if (c->d_bwork) cudaFree(c->d_bwork);
+    if (c->d_nwork) cudaFree(c->d_nwork);
     if (c->own_ws && c->ws) cudaFree(c->ws);
     delete c;
     return LBM_OK;
@@ -2867,6 +3243,7 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
     P.bb = (1.0 - w) / (1.0 - 3.0 * w);
     P.gamma1 = k.gamma1;
     P.gamma2 = k.gamma2;
+    P.bbm2 = -2.0 * P.bb;
     P.omk = 1.0 - P.kk;
     P.k2h = 2.0 * P.kk + P.hh;
     // entries of R without their velocity factors: s_e = 2 ic and s_p = 2 ia,
@@ -2891,6 +3268,7 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
              (kind == lbm::EOS_IDEAL || kind == lbm::EOS_CUBIC) && (long long)k.nx * k.ny >= kModelMinNodes)
                 ? lbm::MODEL_CAVITY
                 : lbm::MODEL_ANY;
+    c->h.mc = c->mc;
     c->h.pd = P;
     convert_params(P, c->h.pf);
     if (!c->tile_set) {
@@ -3051,10 +3429,11 @@ lbm_status lbm_set_tile(lbm_ctx* c, int bx, int by, int pair) {
         CUDA_TRY(cudaStreamSynchronize(c->stream));
         return LBM_OK;
     }
-    if (pair != 0 && pair != 4 && c->cfg.precision != LBM_FP32_DEV)
+    if (pair != 0 && pair != 4 && pair != 6 && c->cfg.precision != LBM_FP32_DEV)
         return fail(LBM_EINVAL, "pair 1-3 and 5 need FP32 storage");
     if (variant_index(bx, pair) < 0)
-        return fail(LBM_EINVAL, pair == 4   ? "warp strips (pair 4) are 30, 60 or 120 columns"
+        return fail(LBM_EINVAL, pair == 6   ? "node kernels (pair 6) take bx = 128"
+                                : pair == 4 ? "warp strips (pair 4) are 30, 60 or 120 columns"
                                 : pair == 5 ? "paired warp strips (pair 5) are 60, 120 or 240 columns"
                                 : (pair == 1 || pair == 2) ? "paired strips (pair 1 or 2) are 64, 128 or 256 columns"
                                                            : "bx must be 32, 64 or 128");
@@ -3086,9 +3465,15 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
     if (nsteps == 0) return LBM_OK;
     const long long base = c->steps;
     CUDA_TRY(cudaMemcpyAsync(c->d_counter, &base, sizeof(base), cudaMemcpyHostToDevice, c->stream));
+    const bool f32 = is_fp32(c);
+    const NWork* prep = c->d_nwork + c->n_node;
+    launch_prep(f32, prep, c->n_prep, c->d_descs, cur_buf(c), 0, nullptr, c->stream);
     for (long s = 0; s < nsteps; ++s) {
         const int par = (int)((c->steps + s) & 1);
-        if (is_fp32(c)) {
+        if (c->n_node) {
+            launch_node(node_kind(c), c->d_nwork, c->n_node, c->d_descs, par, c->d_counter, c->stream);
+            launch_prep(f32, prep, c->n_prep, c->d_descs, par, 1, c->d_counter, c->stream);
+        } else if (f32) {
             launch_collide<float>(c->d_work, c->n_work, variant_index(c->bx, c->pair), c->mc, c->d_descs, par, c->d_counter, c->stream);
             launch_boundary<float>(c->d_bwork, c->n_bwork, c->d_descs, par, c->d_counter, c->stream);
         } else {
@@ -3309,7 +3694,16 @@ lbm_status lbm_conserved_sums_static(const lbm_ctx* c, double* out4) {
 // batched stepping
 // ------------------------------------------------------------------------
 
+// Node kernels: the macros of every member's current buffer, which the
+// first step after this call reads.
+static void batch_launch_first(lbm_batch* b, const LaunchSet& ls, int par, cudaStream_t st) {
+    for (int pr = 0; pr < 2; ++pr)
+        launch_prep(pr == 1, b->d_nwork + ls.p_off[pr], ls.p_cnt[pr], b->d_descs, par, 0, nullptr, st);
+}
+
 static void batch_launch_collide(lbm_batch* b, const LaunchSet& ls, int par, cudaStream_t st) {
+    for (int k = 0; k < kNodeKinds; ++k)
+        launch_node(k, b->d_nwork + ls.n_off[k], ls.n_cnt[k], b->d_descs, par, ls.counter, st);
     for (int pr = 0; pr < 2; ++pr)
         for (int vi = 0; vi < kVariants; ++vi)
             for (int mc = 0; mc < kModels; ++mc) {
@@ -3322,11 +3716,15 @@ static void batch_launch_collide(lbm_batch* b, const LaunchSet& ls, int par, cud
 }
 
 static void batch_launch_boundary(lbm_batch* b, const LaunchSet& ls, int par, cudaStream_t st) {
-    const int last = ls.b_cnt[1] ? 1 : 0;
-    for (int pr = 0; pr < 2; ++pr) {
-        if (!ls.b_cnt[pr]) continue;
-        long long* ctr = (pr == last) ? ls.counter : nullptr;
-        if (pr) launch_boundary<float>(b->d_bwork + ls.b_off[pr], ls.b_cnt[pr], b->d_descs, par, ctr, st);
+    // the last launch of the step advances the step counter
+    int last = -1;
+    for (int k = 0; k < 4; ++k)
+        if (k < 2 ? ls.b_cnt[k] : ls.p_cnt[k - 2]) last = k;
+    for (int k = 0; k < 4; ++k) {
+        const int pr = k & 1;
+        long long* ctr = k == last ? ls.counter : nullptr;
+        if (k >= 2) launch_prep(pr == 1, b->d_nwork + ls.p_off[pr], ls.p_cnt[pr], b->d_descs, par, 1, ctr, st);
+        else if (pr) launch_boundary<float>(b->d_bwork + ls.b_off[pr], ls.b_cnt[pr], b->d_descs, par, ctr, st);
         else launch_boundary<double>(b->d_bwork + ls.b_off[pr], ls.b_cnt[pr], b->d_descs, par, ctr, st);
     }
 }
@@ -3345,7 +3743,26 @@ static lbm_status batch_set_counter(lbm_batch* b) {
 // Launch groups of the members listed in `members` (indices into ctxs) into
 // `ls`, appending their work items to `all` and wall items to `ball`.
 static void build_launch_set(lbm_ctx* const* ctxs, const std::vector<int>& members, int shift, LaunchSet& ls,
-                             std::vector<Work>& all, std::vector<BWork>& ball) {
+                             const std::vector<char>& node, std::vector<Work>& all, std::vector<BWork>& ball,
+                             std::vector<NWork>& nall) {
+    // node kernels: all members' items of one launch together, wall nodes first
+    auto each = [&](auto&& take, auto&& f) {
+        for (int i : members)
+            if (node[i] && take(ctxs[i])) f(i, ctxs[i], (int)(ctxs[i]->steps & 1));
+    };
+    for (int k = 0; k < kNodeKinds; ++k) {
+        ls.n_off[k] = (int)nall.size();
+        each([&](const lbm_ctx* c) { return node_kind(c) == k; },
+             [&](int i, const lbm_ctx* c, int par) { add_node_work(c->cfg, i, par, k == kNodePair, c->steps, nall); });
+        ls.n_cnt[k] = (int)nall.size() - ls.n_off[k];
+    }
+    for (int pr = 0; pr < 2; ++pr) {
+        auto mine = [&](const lbm_ctx* c) { return is_fp32(c) == (pr == 1); };
+        ls.p_off[pr] = (int)nall.size();
+        each(mine, [&](int i, const lbm_ctx* c, int par) { add_prep_wall(c->cfg, i, par, nall); });
+        each(mine, [&](int i, const lbm_ctx* c, int par) { add_prep_inner(c->cfg, i, par, nall); });
+        ls.p_cnt[pr] = (int)nall.size() - ls.p_off[pr];
+    }
     std::vector<Work> groups[2][kVariants][kModels];
     std::vector<BWork> bgroups[2];
     // Members with longer runs first, and each member's runs together in
@@ -3365,6 +3782,7 @@ static void build_launch_set(lbm_ctx* const* ctxs, const std::vector<int>& membe
     std::vector<int> order(members);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return run_len(a) > run_len(b); });
     for (int i : order) {
+        if (node[i]) continue;
         const lbm_ctx* c = ctxs[i];
         const int pr = is_fp32(c) ? 1 : 0, bi = variant_index(c->bx, c->pair);
         const int par = (int)(c->steps & 1);
@@ -3373,6 +3791,7 @@ static void build_launch_set(lbm_ctx* const* ctxs, const std::vector<int>& membe
         grp.insert(grp.end(), w.begin(), w.end());
     }
     for (int i : members) {
+        if (node[i]) continue;
         const lbm_ctx* c = ctxs[i];
         auto bw = make_bwork(c->cfg, i, (int)(c->steps & 1));
         bgroups[is_fp32(c) ? 1 : 0].insert(bgroups[is_fp32(c) ? 1 : 0].end(), bw.begin(), bw.end());
@@ -3387,7 +3806,7 @@ static void build_launch_set(lbm_ctx* const* ctxs, const std::vector<int>& membe
                 ls.w_cnt[pr][bi][mc] = (int)g.size();
                 all.insert(all.end(), g.begin(), g.end());
             }
-    if (bgroups[0].empty() && bgroups[1].empty()) {
+    if (bgroups[0].empty() && bgroups[1].empty() && !ls.p_cnt[0] && !ls.p_cnt[1]) {
         const lbm_ctx* c = ctxs[members[0]];
         ensure_tick(bgroups[is_fp32(c) ? 1 : 0], members[0], (int)(c->steps & 1));
     }
@@ -3406,6 +3825,11 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int n, int graph_steps, lbm_ba
     lbm_batch* b = new lbm_batch();
     b->stream = ctxs[0]->stream;
     std::vector<InstDesc*> descs;
+    long long nodes32 = 0;  // FP32 members with a default shape
+    for (int i = 0; i < n; ++i)
+        if (ctxs[i] && !ctxs[i]->tile_set && is_fp32(ctxs[i])) nodes32 += (long long)ctxs[i]->cfg.nx * ctxs[i]->cfg.ny;
+    std::vector<char> node(n, 0);
+    for (int i = 0; i < n; ++i) node[i] = ctxs[i] && node_kernels(ctxs[i], nodes32);
     // rows per run of the members whose shape was not set: the batch length,
     // halved for all of them while the batch fills less than the GPU once
     // (each CTA of a member takes 1 / resident_ctas of the GPU)
@@ -3415,7 +3839,7 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int n, int graph_steps, lbm_ba
         bool can_halve = false;
         for (int i = 0; i < n; ++i) {
             const lbm_ctx* c = ctxs[i];
-            if (!c || c->tile_set) continue;
+            if (!c || c->tile_set || node[i]) continue;
             const int by = std::max(1, batch_rows(c->cfg, c->pair) >> shift);
             can_halve = can_halve || by > 1;
             fill += (double)cta_count(c->cfg, c->bx, by) /
@@ -3435,9 +3859,10 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int n, int graph_steps, lbm_ba
     }
     std::vector<Work> all;
     std::vector<BWork> ball;
+    std::vector<NWork> nall;
     std::vector<int> everyone(n);
     for (int i = 0; i < n; ++i) everyone[i] = i;
-    build_launch_set(ctxs, everyone, shift, b->set, all, ball);
+    build_launch_set(ctxs, everyone, shift, b->set, node, all, ball, nall);
     auto bad = [&](const char* m) {
         lbm_batch_destroy(b);
         return fail(LBM_ECUDA, m);
@@ -3448,12 +3873,15 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int n, int graph_steps, lbm_ba
     b->set.counter = b->d_counter;
     if (!all.empty() && cudaMalloc(&b->d_work, all.size() * sizeof(Work)) != cudaSuccess) return bad("cudaMalloc work");
     if (!ball.empty() && cudaMalloc(&b->d_bwork, ball.size() * sizeof(BWork)) != cudaSuccess) return bad("cudaMalloc bwork");
+    if (!nall.empty() && cudaMalloc(&b->d_nwork, nall.size() * sizeof(NWork)) != cudaSuccess) return bad("cudaMalloc node work");
     if (cudaMemcpyAsync(b->d_descs, descs.data(), descs.size() * sizeof(InstDesc*), cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
         return bad("upload descs");
     if (!all.empty() && cudaMemcpyAsync(b->d_work, all.data(), all.size() * sizeof(Work), cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
         return bad("upload work");
     if (!ball.empty() && cudaMemcpyAsync(b->d_bwork, ball.data(), ball.size() * sizeof(BWork), cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
         return bad("upload bwork");
+    if (!nall.empty() && cudaMemcpyAsync(b->d_nwork, nall.data(), nall.size() * sizeof(NWork), cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
+        return bad("upload node work");
     if (cudaStreamSynchronize(b->stream) != cudaSuccess) return bad("sync");
     b->graph_steps = graph_steps;
     if (graph_steps > 0) {
@@ -3515,8 +3943,10 @@ lbm_status lbm_batch_step(lbm_batch* b, long nsteps) {
     if (cs != LBM_OK) return cs;
     if (b->graph) {
         if (nsteps % b->graph_steps) return fail(LBM_EINVAL, "nsteps must be a multiple of graph_steps");
+        batch_launch_first(b, b->set, 0, b->stream);
         for (long s = 0; s < nsteps; s += b->graph_steps) CUDA_TRY(cudaGraphLaunch(b->graph, b->stream));
     } else {
+        batch_launch_first(b, b->set, (int)(b->steps & 1), b->stream);
         for (long s = 0; s < nsteps; ++s) batch_launch_step(b, b->set, (int)((b->steps + s) & 1), b->stream);
         lbm_status st = check_launch();
         if (st != LBM_OK) return st;
@@ -3542,6 +3972,7 @@ lbm_status lbm_batch_step_profiled(lbm_batch* b, long nsteps, double* ms_collide
         if (cudaEventCreate(&e) != cudaSuccess) { cleanup(); return fail(LBM_ECUDA, "cudaEventCreate"); }
     lbm_status cs = batch_set_counter(b);
     if (cs != LBM_OK) { cleanup(); return cs; }
+    batch_launch_first(b, b->set, (int)(b->steps & 1), b->stream);
     for (long s = 0; s < nsteps; ++s) {
         const int par = (int)((b->steps + s) & 1);
         cudaEventRecord(ev[3 * s], b->stream);
@@ -3693,6 +4124,7 @@ lbm_status lbm_batch_destroy(lbm_batch* b) {
     if (b->d_descs) cudaFree(b->d_descs);
     if (b->d_work) cudaFree(b->d_work);
     if (b->d_bwork) cudaFree(b->d_bwork);
+    if (b->d_nwork) cudaFree(b->d_nwork);
     delete b;
     return LBM_OK;
 }

@@ -15,6 +15,13 @@
 //  G = (I - S/2) d and C = R G + T grad(rho) + X grad(p),
 //  L applied as diag(L) plus the two sigma_q omega_j couplings (Sec. 2.2),
 //  M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4).
+//
+// Every fused multiply-add is written as mad() and the library is compiled
+// without the compiler's own contraction (-fmad=false), so a node's bits
+// depend on its inputs alone: all kernels, scalar or packed, that update a
+// lattice give the same state.  A product with a literal constant that meets
+// an addition is always a mad(): the assembler contracts the packed form of
+// that pair of instructions all the same.
 #pragma once
 
 #include <cmath>
@@ -120,7 +127,7 @@ struct Params {
     R mu0, mu0S, inv_T0, visc_S, lam_fac;
     R nu_e, mu_j;     // 2 * 3 varsigma / (varpi nu), 2 (1/sigma_j - 1/2) / mu (Rates)
     R beta2;          // -2 beta1 / (1 - varpi); alpha1 = -1, beta1 = 1, alpha2 = 1 are fixed
-    R kk, hh, bb, omk, k2h, gamma1, gamma2;
+    R kk, hh, bb, bbm2, omk, k2h, gamma1, gamma2;  // bbm2 = -2 bb
     R k11, k17, k18, k71, k77, k81, k88;  // entries of R per 1/(1 + 6 nu) or 1/(1 + nu_e nu) (collide)
     R Fx, Fy;
     R cs_b0;  // 1 - b rho0 (cubic EOS)
@@ -163,12 +170,14 @@ struct MacC {
 // Carnahan-Starling deviation p - p0 with p = Z(e) rho R T, e = b rho / 4
 // (Eq. EOSs.3).  The density part is differenced in FP64 to avoid
 // cancellation when the arithmetic type is FP32.
+LBM_HD double cs_z(double e) {  // Z = (1 + e + e^2 - e^3) / (1 - e)^3
+    const double om = 1.0 - e;
+    return fdiv(mad(mad(mad(-1.0, e, 1.0), e, 1.0), e, 1.0), om * om * om);
+}
 LBM_HD double cs_dev1(double b, double rho0, double Rg, double rho_d, double T, double T_d) {
-    double r = rho0 + rho_d;
-    double e = b * r / 4.0, e0 = b * rho0 / 4.0;
-    double z = (1.0 + e + e * e - e * e * e) / ((1.0 - e) * (1.0 - e) * (1.0 - e));
-    double z0 = (1.0 + e0 + e0 * e0 - e0 * e0 * e0) / ((1.0 - e0) * (1.0 - e0) * (1.0 - e0));
-    return Rg * ((z * r - z0 * rho0) * T + z0 * rho0 * T_d);
+    const double r = rho0 + rho_d;
+    const double z0r = cs_z(0.25 * b * rho0) * rho0;
+    return Rg * mad(mad(cs_z(0.25 * b * r), r, -z0r), T, z0r * T_d);
 }
 LBM_HD double cs_dev(double b, double rho0, double Rg, double rho_d, double T, double T_d) {
     return cs_dev1(b, rho0, Rg, rho_d, T, T_d);
@@ -181,20 +190,20 @@ LBM_HD float cs_dev(float b, float rho0, float Rg, float rho_d, float T, float T
 template <int MC = MODEL_ANY, typename R>
 LBM_HD R eos_dev(const Params<R>& P, R rho_d, R rho, R T_d, R T) {
     const int kind = MC == MODEL_CAVITY ? (P.eos == EOS_CUBIC ? EOS_CUBIC : EOS_IDEAL) : P.eos;
-    if (MC == MODEL_CAVITY && kind == EOS_IDEAL) return P.Rg * (rho_d * T + P.rho0 * T_d);
+    if (MC == MODEL_CAVITY && kind == EOS_IDEAL) return P.Rg * mad(rho_d, T, P.rho0 * T_d);
     switch (kind) {
     case EOS_DECOUPLING:
         return P.Rg * P.T0 * rho_d;
     case EOS_IDEAL:
-        return P.Rg * (rho_d * T + P.rho0 * T_d);
+        return P.Rg * mad(rho_d, T, P.rho0 * T_d);
     case EOS_CS:
         return cs_dev(P.eos_b, P.rho0, P.Rg, rho_d, T, T_d);
     default: {
         // rho R T / (1 - b rho) - a rho^2, differenced exactly:
-        // [rho T (1 - b rho0) - rho0 T0 (1 - b rho)] = rho_d T + rho0 T_d - b rho rho0 T_d
-        R om = R(1) - P.eos_b * rho;
-        R num = rho_d * T + P.rho0 * T_d - P.eos_b * rho * P.rho0 * T_d;
-        return fdiv(P.Rg * num, om * P.cs_b0) - P.eos_a * rho_d * (rho + P.rho0);
+        // [rho T (1 - b rho0) - rho0 T0 (1 - b rho)] = rho_d T + rho0 T_d (1 - b rho)
+        const R om = mad(-P.eos_b, rho, R(1));
+        const R num = mad(rho_d, T, P.rho0 * T_d * om);
+        return mad(-P.eos_a * rho_d, rho + P.rho0, fdiv(P.Rg * num, om * P.cs_b0));
     }
     }
 }
@@ -267,14 +276,13 @@ LBM_HD void wall_macros(const Params<R>& P, R rho_d, R ux, R uy, R rhoE_d, Mac<R
     m.rho_d = rho_d;
     m.rho = P.rho0 + rho_d;
     m.ir = recip(m.rho);
-    if (P.force_mode) { m.Fx = m.rho * P.Fx; m.Fy = m.rho * P.Fy; }
-    else { m.Fx = P.Fx; m.Fy = P.Fy; }
+    mac_force(P, m);
     m.ux = ux;
     m.uy = uy;
-    m.qe = ux * m.Fx + uy * m.Fy;
+    mac_qe(m);
     m.rhoE_d = rhoE_d;
-    R E_d = (rhoE_d - rho_d * P.E0) * m.ir;
-    m.T_d = (E_d - R(0.5) * (ux * ux + uy * uy)) * P.inv_Cv;
+    R E_d = mad(-P.E0, rho_d, rhoE_d) * m.ir;
+    m.T_d = mad(R(-0.5), mad(ux, ux, uy * uy), E_d) * P.inv_Cv;
     m.T = P.T0 + m.T_d;
     m.p_d = eos_dev(P, rho_d, m.rho, m.T_d, m.T);
     mac_tail(P, m);
@@ -343,19 +351,19 @@ LBM_HD void neq_density(const Params<R>& P, const Mac<R>& m, R m1, R m2, R m4, R
     d.x6 = mad(-t3, ux, m6 + jy);
     d.x7 = mad(jy, uy, m7 - jxx);
     d.x8 = m8 - jxy;
-    const R Fx = m.Fx, Fy = m.Fy, q3 = R(3) * m.qe;
-    d.d1 = d.x1 + q3;
+    const R Fx = m.Fx, Fy = m.Fy;
+    d.d1 = mad(R(3), m.qe, d.x1);
     if (MC == MODEL_CAVITY) {
         // the same terms with F_x = 0
         const R w = mad(R(3), ux * ux, R(-1)), Fh = R(0.5) * Fy;
-        d.d2 = mad(q3, w, d.x2);
+        d.d2 = mad(R(3) * m.qe, w, d.x2);
         d.d4 = mad(R(3) * Fy, xy, d.x4);
         d.d6 = mad(Fh, w, d.x6);
         d.d7 = d.x7 - m.qe;
         d.d8 = mad(Fh, ux, d.x8);
     } else {
         const R s8 = mad(Fx, uy, Fy * ux), xy3 = R(3) * xy;
-        d.d2 = mad(R(3) * xy3, s8, d.x2 - q3);
+        d.d2 = mad(R(3) * xy3, s8, mad(R(-3), m.qe, d.x2));
         d.d4 = mad(xy3, Fy, mad(R(0.5) * Fx, mad(R(3), uy * uy, R(-1)), d.x4));
         d.d6 = mad(xy3, Fx, mad(R(0.5) * Fy, mad(R(3), ux * ux, R(-1)), d.x6));
         d.d7 = mad(-Fy, uy, mad(Fx, ux, d.x7));
@@ -474,6 +482,14 @@ LBM_HD void gradient3(R ml, R mc, R mr, R zl, R zr, R pl, R pc, R pr, R& gx, R& 
     gy = mad(R(0.25), a - b, pc - mc);
 }
 
+// Three times a one-sided second-order derivative along the inward normal
+// (s = 1 towards increasing coordinates, -1 otherwise) at a wall node, and
+// three times a central one along a wall.
+template <typename R>
+LBM_HD R onesided3(R s, R v0, R v1, R v2) { return s * R(1.5) * mad(R(4), v1, mad(R(-3), v0, -v2)); }
+template <typename R>
+LBM_HD R central3(R l, R r) { return R(1.5) * (r - l); }
+
 // Full collision of one node (Eqs. LBE.u.c, LBE.T.c) in increment form: the
 // moment changes m_bar - m and n_bar - n are formed from small quantities
 // only (force and source moments, non-equilibrium parts, corrections), then
@@ -513,15 +529,15 @@ LBM_HD void collide(const Params<R>& P, const Mac<R>& mc, R* f, R* g, R rx, R ry
     R Gt1 = G.G1, Gt7 = G.G7, Gt8 = G.G8;
     if (corrections_on<MC>(P)) {
         const R ux2 = ux * ux, uy2 = uy * uy, sum2 = ux2 + uy2, dif2 = ux2 - uy2, xy = ux * uy;
-        const R he = R(1) - r.ic, hp = R(1) - r.ia;
+        const R he = R(1) - r.ic, hp3 = R(1.0 / 3.0) * (R(1) - r.ia);
         const R zx = mad(R(3), px, -rx), zy = mad(R(3), py, -ry);
         const R p1 = ux2 * (ux * rx), p2 = uy2 * (uy * ry), p3 = uy2 * (ux * zx), p4 = ux2 * (uy * zy);
         const R C1 = mad(he, mad(P.omk, p1 + p2, P.k2h * (p3 + p4)),
                          r.ic * mad(P.k11, sum2 * G.G1, mad(P.k17, dif2 * G.G7, P.k18 * (xy * G.G8))));
-        const R C7 = mad(hp, mad(R(-2.0 / 3.0) * P.bb, p3 - p4, R(1.0 / 3.0) * (p1 - p2)),
+        const R C7 = mad(hp3, mad(P.bbm2, p3 - p4, p1 - p2),
                          r.ia * mad(P.k71, dif2 * G.G1, P.k77 * (sum2 * G.G7)));
         const R v8 = mad(mad(R(2), ux2, uy2), uy * zx, mad(R(2), uy2, ux2) * (ux * zy));
-        const R C8 = mad(R(1.0 / 3.0) * P.bb * hp, v8, r.ia * mad(P.k81, xy * G.G1, P.k88 * (sum2 * G.G8)));
+        const R C8 = mad(P.bb * hp3, v8, r.ia * mad(P.k81, xy * G.G1, P.k88 * (sum2 * G.G8)));
         Gt1 = mad(R(-0.5), C1, Gt1);
         Gt7 = mad(R(-0.5), C7, Gt7);
         Gt8 = mad(R(-0.5), C8, Gt8);

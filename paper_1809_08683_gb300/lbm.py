@@ -20,7 +20,7 @@ _DEPS = [_SRC, os.path.join(_HERE, "csrc", "lbm_node.cuh"), os.path.join(_HERE, 
          os.path.join(_HERE, "csrc", "lbm_ff.cuh"), os.path.join(os.path.dirname(_HERE), "include", "lbm.h")]
 _BUILD = os.path.join(_HERE, "_build")
 LIB_PATH = os.path.join(_BUILD, "liblbm_gb300.so")
-NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo",
+NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo", "-fmad=false",
               "-Xcompiler", "-fPIC", "-shared"]
 
 LBM_OK, LBM_EINVAL, LBM_ENOMEM, LBM_ECUDA, LBM_EUNSTABLE, LBM_ETIMEOUT = 0, -1, -2, -3, -4, -5
