@@ -332,14 +332,12 @@ def serving_run(n, n_compare, sides=(24, 96)):
 def steady_cavity512(tol=1e-8):
     """The 512^2 heated cavity at Ra = 1e6, eps = 0.6, ideal gas,
     Sutherland viscosity, run from rest to residual `tol` in FP32 deviation
-    storage, finished in FP64 once FP32 stalls; its lone launch shape from
-    the autotuner.  Nu_ave and p*_ave against Table 2."""
-    from paper_1809_08683_gb300 import autotune, serve
+    storage, finished in FP64 once FP32 stalls, in the default launch shape
+    (node kernels in both precisions).  Nu_ave and p*_ave against Table 2."""
+    from paper_1809_08683_gb300 import serve
     cfg = W.cavity(N=512, Ra=1e6, eps=0.6, precision=1)
     req = serve.Request(rid=0, cfg=cfg, tol=tol, max_steps=3_000_000)
-    srv = serve.Server(max_slots=1, chunk=1000, graph_steps=1000, tile_fn=lambda c: autotune.tune(c, steps=10))
-    for prec in (1, 0):                 # tune outside the timed solve
-        autotune.tune(dict(cfg, precision=prec), steps=10)
+    srv = serve.Server(max_slots=1, chunk=1000, graph_steps=1000)
     srv.run([req], realtime=False)
     nu, ps = req.result.get("nusselt"), req.result.get("pstar")
     return {"workload": "cavity_512x512_Ra1e6_eps0.6", "tol": tol, "status": req.status, "s": req.latency,

@@ -58,15 +58,16 @@ WARP2_BX_CANDIDATES = (60, 120, 240)
 
 
 def candidates(cfg: dict):
-    """(bx, by, pair) shapes worth timing for this lattice: one node per
+    """(bx, by, pair) strip shapes worth timing for this lattice: one node per
     thread in block strips or warp strips for every precision, two nodes per
-    thread for FP32 storage."""
+    thread for FP32 storage.  A lattice whose shape is not set steps through
+    the node kernels where those are faster (FP64, and small FP32 lattices)."""
     shapes = [(bx, 0) for bx in BX_CANDIDATES] + [(bx, 4) for bx in WARP_BX_CANDIDATES]
     if int(cfg.get("precision", 0)) == 1:
         shapes += [(bx, 3) for bx in BX_CANDIDATES]
         shapes += [(bx, pr) for bx in PAIR_BX_CANDIDATES for pr in (1, 2)]
         shapes += [(bx, 5) for bx in WARP2_BX_CANDIDATES]
-    out = [(128, 1, 6)]   # node kernels: one node per thread over the whole lattice
+    out = []
     for bx, pr in shapes:
         if bx > 32 and cfg["nx"] <= bx // 2:
             continue
@@ -78,9 +79,8 @@ def candidates(cfg: dict):
 
 
 def measure(cfg: dict, bx: int, by: int, pair: int = 0, steps: int = 20, stream=None) -> float:
-    """MLUPS of whole steps (the collision and the wall pass) for one launch
-    shape; the two cannot be told apart across shapes, since the node kernels
-    form the macros of a step in the launch that rebuilds the wall nodes."""
+    """MLUPS of whole steps (the fused launch and the wall pass) for one
+    launch shape."""
     lat = lbm.Lattice(cfg, stream=stream)
     lat.set_tile(bx, by, pair)
     batch = lbm.Batch([lat], graph_steps=0)
