@@ -2047,27 +2047,92 @@ __global__ void k_copy_state(const Rs* __restrict__ src, long long splane, int s
     }
 }
 
+// FP64 sums over the populations of a node stored in FP32.  An FP64 addition
+// or FP32-to-FP64 conversion issues once per 76 cycles and scheduler, and 18
+// conversions and 24 additions were most of what the readers of the state
+// spent.  Instead the sums are formed exactly in 64-bit integers: with the
+// largest exponent emax of the nine values, each is its signed 24-bit
+// mantissa times 2^(e - emax + 30), one wide multiply-add per term, and the
+// sum is converted, and so rounded, once.  Values more than 30 binades below
+// the largest, denormals, infinities and NaN take the FP64 additions.
+// k_macros with its consumer's passes, 39.2M nodes: 6.3 -> 3.5 ms.
+struct Fixed9 {
+    int m[9], p[9];  // mantissa with sign, power of two
+    int emax;
+    __device__ __forceinline__ bool set(const float* f) {
+        int e[9];
+        emax = 0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            e[i] = (__float_as_int(f[i]) >> 23) & 255;
+            emax = max(emax, e[i]);
+        }
+        bool ok = emax != 255;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const int b = __float_as_int(f[i]), s = b >> 31;
+            const bool zero = (b & 0x7fffffff) == 0;
+            const int sh = e[i] - emax + 30;
+            ok = ok && (zero || (e[i] != 0 && sh >= 0));
+            m[i] = zero ? 0 : ((((b & 0x007fffff) | 0x00800000) ^ s) - s);
+            p[i] = 1 << (sh & 31);
+        }
+        return ok;
+    }
+    __device__ __forceinline__ long long at(int i) const { return (long long)m[i] * p[i]; }
+    // the sum v of terms at(i), scaled back
+    __device__ __forceinline__ double value(long long v) const {
+        if (v == 0) return 0.0;
+        const double d = (double)v;  // times 2^(emax - 180), by its exponent field
+        return __hiloint2double(__double2hiint(d) + ((emax - 180) << 20), __double2loint(d));
+    }
+};
+
+__device__ __forceinline__ void node_sums_fp64(const double* v, double& rd, double& jx, double& jy, double& sg) {
+    lbm::node_sums(v, v + 9, rd, jx, jy, sg);
+}
+__device__ __forceinline__ void node_sums_fp64(const float* v, double& rd, double& jx, double& jy, double& sg) {
+    Fixed9 f, g;
+    const bool okf = f.set(v), okg = g.set(v + 9);
+    if (okf && okg) {
+        const long long d1 = f.at(5) - f.at(7), d2 = f.at(6) - f.at(8);
+        long long r = f.at(0), s = g.at(0);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            r += f.at(i);
+            s += g.at(i);
+        }
+        rd = f.value(r);
+        jx = f.value(f.at(1) - f.at(3) + (d1 - d2));
+        jy = f.value(f.at(2) - f.at(4) + (d1 + d2));
+        sg = g.value(s);
+    } else {
+        double w[18];
+#pragma unroll
+        for (int q = 0; q < 18; ++q) w[q] = (double)v[q];
+        lbm::node_sums(w, w + 9, rd, jx, jy, sg);
+    }
+}
+
 // FP64 macros of one node of an R-typed buffer.
 template <typename R>
 __device__ __forceinline__ void macros_fp64(const InstDesc* D, const R* buf, int x, int y, Mac<double>& m) {
     R v[18];
     load18(buf, D->plane, (long long)y * D->pitch + x, v);
-    double w[18];
-#pragma unroll
-    for (int q = 0; q < 18; ++q) w[q] = (double)v[q];
     double rd, jx, jy, sg;
-    lbm::node_sums(w, w + 9, rd, jx, jy, sg);
+    node_sums_fp64(v, rd, jx, jy, sg);
     lbm::macros(D->pd, rd, jx, jy, sg, m);
 }
 
+constexpr int kMacroThreads = 128;
 template <typename R>
-__global__ void k_macros(const InstDesc* D, int b, double* rho, double* ux, double* uy, double* T,
-                         double* p) {
+__global__ void __launch_bounds__(kMacroThreads) k_macros(const InstDesc* D, int b, double* rho, double* ux, double* uy,
+                                                         double* T, double* p) {
     const long long nn = (long long)D->nx * D->ny;
     const R* buf = reinterpret_cast<const R*>(D->buf[b]);
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nn;
          t += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(t / D->nx), x = (int)(t % D->nx);
+        const int y = (int)t / D->nx, x = (int)t - y * D->nx;  // t < 2^31: checked at creation
         Mac<double> m;
         macros_fp64(D, buf, x, y, m);
         if (rho) rho[t] = m.rho;
@@ -2079,8 +2144,19 @@ __global__ void k_macros(const InstDesc* D, int b, double* rho, double* ux, doub
 }
 
 constexpr int kDiagSlots = 10;
-constexpr int kDiagBlocks = 304;   // 2 per SM on a 152-SM part; fixed for a deterministic order
+constexpr int kDiagBlocks = 304;      // 2 per SM on a 152-SM part; fixed for a deterministic order
 constexpr int kDiagThreads = 256;
+constexpr int kDiagNodesPerBlock = 512;
+
+// Blocks of the diagnostics of a lattice of nn nodes, alone or batched: a
+// block's reduction costs as many FP64 instructions as three nodes per
+// thread, so a small lattice takes few (with 304 for every lattice the
+// reductions were 662 of the FP64 additions per node of 64 small lattices:
+// 0.65 ms against 0.07 ms for the nodes themselves).
+__host__ __device__ inline int diag_blocks(long long nn) {
+    const long long b = (nn + kDiagNodesPerBlock - 1) / kDiagNodesPerBlock;
+    return (int)(b < kDiagBlocks ? b : kDiagBlocks);
+}
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -2088,67 +2164,81 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// Larger of two non-negative numbers (their bits order like integers; an
+// FP64 comparison would take an FP64 issue slot).
+__device__ __forceinline__ double max_nonneg(double a, double b) {
+    return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+}
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
+    for (int o = 16; o > 0; o >>= 1) v = max_nonneg(v, __shfl_down_sync(0xffffffffu, v, o));
     return v;
 }
 
-// Per-block FP64 partial sums (slot 8 is a maximum) into partials[block][kDiagSlots]:
-// block blk of nblk, grid-stride over the lattice's nodes.  k_diag and the
-// batched k_diag_batch run this with the same decomposition, so a lattice's
-// diagnostics are the same bits alone or batched.
+// Per-block FP64 partial sums into partials[block][kDiagSlots]: block blk of
+// nblk, grid-stride over the lattice's nodes.  k_diag and the batched
+// k_diag_batch run this with the same decomposition, so a lattice's
+// diagnostics are the same bits alone or batched.  Slots: 0 rho', 1 (rho E)',
+// 2 p' with half weights on the walls, 3 |du|^2, 4 |u|^2, 5 dT^2, 6 T'^2,
+// 7 non-finite nodes, 8 maximum of |u|^2, 9 T'.
 template <typename R>
 __device__ __forceinline__ void diag_partials(const InstDesc* D, int b, double* __restrict__ snap, int take_snapshot,
                                               int have_snapshot, double* __restrict__ partials, int blk, int nblk) {
-    const long long nn = (long long)D->nx * D->ny;
+    const int nx = D->nx, ny = D->ny;
+    const long long nn = (long long)nx * ny;
     const R* buf = reinterpret_cast<const R*>(D->buf[b]);
     double acc[kDiagSlots];
 #pragma unroll
     for (int s = 0; s < kDiagSlots; ++s) acc[s] = 0.0;
-    const double Lx = D->px ? (double)D->nx : (double)(D->nx - 1);
-    const double Ly = D->py ? (double)D->ny : (double)(D->ny - 1);
+    int bad = 0;
     for (long long t = blk * (long long)blockDim.x + threadIdx.x; t < nn; t += (long long)nblk * blockDim.x) {
-        const int y = (int)(t / D->nx), x = (int)(t % D->nx);
+        const int y = (int)t / nx, x = (int)t - y * nx;
         Mac<double> m;
         macros_fp64(D, buf, x, y, m);
-        const bool bad = !(isfinite(m.rho) && isfinite(m.T) && isfinite(m.ux) && isfinite(m.uy));
-        if (bad) { acc[7] += 1.0; continue; }
-        const double wx = (!D->px && (x == 0 || x == D->nx - 1)) ? 0.5 : 1.0;
-        const double wy = (!D->py && (y == 0 || y == D->ny - 1)) ? 0.5 : 1.0;
-        const double p = D->pd.p0 + m.p_d;
+        const bool edge_x = !D->px && (x == 0 || x == nx - 1), edge_y = !D->py && (y == 0 || y == ny - 1);
+        if (!(lbm::finite(m.rho) && lbm::finite(m.T) && lbm::finite(m.ux) && lbm::finite(m.uy))) {
+            // counts as zero pressure and temperature
+            ++bad;
+            acc[2] -= (edge_x ? 0.5 : 1.0) * (edge_y ? 0.5 : 1.0) * D->pd.p0;
+            acc[9] -= D->pd.T0;
+            continue;
+        }
         acc[0] += m.rho_d;
         acc[1] += m.rhoE_d;
-        acc[2] += wx * wy * p / (D->pd.p0 * Lx * Ly);
+        if (edge_x || edge_y) acc[2] = lbm::mad(edge_x && edge_y ? 0.25 : 0.5, m.p_d, acc[2]);
+        else acc[2] += m.p_d;
         const double u2 = lbm::mad(m.ux, m.ux, m.uy * m.uy);
         if (have_snapshot) {
             const double dux = m.ux - snap[t], duy = m.uy - snap[nn + t], dT = m.T - snap[2 * nn + t];
-            acc[3] += lbm::mad(dux, dux, duy * duy);
+            acc[3] = lbm::mad(dux, dux, lbm::mad(duy, duy, acc[3]));
             acc[5] = lbm::mad(dT, dT, acc[5]);
         }
         acc[4] += u2;
         acc[6] = lbm::mad(m.T_d, m.T_d, acc[6]);
-        acc[8] = fmax(acc[8], sqrt(u2));
-        acc[9] += m.T;
+        acc[8] = max_nonneg(acc[8], u2);
+        acc[9] += m.T_d;
         if (take_snapshot) {
             snap[t] = m.ux;
             snap[nn + t] = m.uy;
             snap[2 * nn + t] = m.T;
         }
     }
-    __shared__ double red[kDiagThreads / 32][kDiagSlots];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    acc[7] = (double)bad;
+    // The block's sums: every thread's slots through shared memory, then one
+    // warp per slot (12 FP64 instructions a slot, against 5 a slot and warp
+    // with shuffles alone).
+    constexpr int kWarps = kDiagThreads / 32;
+    __shared__ double red[kDiagSlots][kDiagThreads];
 #pragma unroll
-    for (int s = 0; s < kDiagSlots; ++s) {
-        const double v = (s == 8) ? warp_max(acc[s]) : warp_sum(acc[s]);
-        if (lane == 0) red[wid][s] = v;
-    }
+    for (int s = 0; s < kDiagSlots; ++s) red[s][threadIdx.x] = acc[s];
     __syncthreads();
-    if (threadIdx.x < kDiagSlots) {
-        const int s = threadIdx.x;
-        double v = red[0][s];
-        for (int k = 1; k < kDiagThreads / 32; ++k) v = (s == 8) ? fmax(v, red[k][s]) : v + red[k][s];
-        partials[blk * kDiagSlots + s] = v;
+    const int lane = threadIdx.x & 31;
+    for (int s = threadIdx.x >> 5; s < kDiagSlots; s += kWarps) {
+        double v = red[s][lane];
+#pragma unroll
+        for (int k = 1; k < kWarps; ++k) v = (s == 8) ? max_nonneg(v, red[s][lane + 32 * k]) : v + red[s][lane + 32 * k];
+        v = (s == 8) ? warp_max(v) : warp_sum(v);
+        if (lane == 0) partials[blk * kDiagSlots + s] = v;
     }
 }
 
@@ -2159,41 +2249,50 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag(const InstDesc* D, int b,
     diag_partials<R>(D, b, snap, take_snapshot, have_snapshot, partials, blockIdx.x, gridDim.x);
 }
 
-// One lattice of a batched diagnostics pass (lbm_batch_diagnostics).
+// One lattice of a diagnostics pass, and the first of its blocks in a
+// batched one.
 struct DiagJob {
     const InstDesc* D;
     double* snap;
     double* partials;
     const unsigned int* status;
-    int b, have;
+    int b, have, first_block, nblocks;
 };
 
-// Every lattice of one storage precision at once: blockIdx.y picks the job.
+// Every lattice of one storage precision at once: the job whose blocks hold
+// blockIdx.x, by bisection.
 template <typename R>
-__global__ void __launch_bounds__(kDiagThreads) k_diag_batch(const DiagJob* __restrict__ jobs, int take_snapshot) {
-    const DiagJob j = jobs[blockIdx.y];
-    diag_partials<R>(j.D, j.b, j.snap, take_snapshot, j.have, j.partials, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(kDiagThreads) k_diag_batch(const DiagJob* __restrict__ jobs, int njobs, int take_snapshot) {
+    int lo = 0, hi = njobs;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (jobs[mid].first_block <= (int)blockIdx.x) lo = mid;
+        else hi = mid;
+    }
+    const DiagJob j = jobs[lo];
+    diag_partials<R>(j.D, j.b, j.snap, take_snapshot, j.have, j.partials, blockIdx.x - j.first_block, j.nblocks);
 }
 
-__global__ void k_diag_final(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
-    const int s = threadIdx.x;
-    if (s >= kDiagSlots) return;
+// The sums of a lattice's kDiagSlots, then its status word, into out
+// [kDiagSlots + 1]: one warp per slot, lanes striding over the blocks.
+__device__ __forceinline__ void diag_final(const double* __restrict__ partials, int nblocks, const unsigned int* status, double* out) {
+    const int lane = threadIdx.x & 31, s = threadIdx.x >> 5;
     double v = 0.0;
-    for (int k = 0; k < nblocks; ++k) v = (s == 8) ? fmax(v, partials[k * kDiagSlots + s]) : v + partials[k * kDiagSlots + s];
-    out[s] = v;
+    for (int k = lane; k < nblocks; k += 32) {
+        const double u = partials[k * kDiagSlots + s];
+        v = (s == 8) ? max_nonneg(v, u) : v + u;
+    }
+    v = (s == 8) ? warp_max(v) : warp_sum(v);
+    if (lane == 0) out[s] = v;
+    if (threadIdx.x == 0) out[kDiagSlots] = (double)*status;
 }
-
-// Block b finishes job b: its kDiagSlots sums, then its status word, into
-// out[b][kDiagSlots + 1], in the order k_diag_final uses.
-__global__ void k_diag_final_batch(const DiagJob* __restrict__ jobs, int nblocks, double* __restrict__ out) {
+__global__ void __launch_bounds__(32 * kDiagSlots) k_diag_final(const double* __restrict__ partials, int nblocks,
+                                                               const unsigned int* status, double* __restrict__ out) {
+    diag_final(partials, nblocks, status, out);
+}
+__global__ void __launch_bounds__(32 * kDiagSlots) k_diag_final_batch(const DiagJob* __restrict__ jobs, double* __restrict__ out) {
     const DiagJob j = jobs[blockIdx.x];
-    const int s = threadIdx.x;
-    double* o = out + (size_t)blockIdx.x * (kDiagSlots + 1);
-    if (s == kDiagSlots) o[s] = (double)*j.status;
-    if (s >= kDiagSlots) return;
-    double v = 0.0;
-    for (int k = 0; k < nblocks; ++k) v = (s == 8) ? fmax(v, j.partials[k * kDiagSlots + s]) : v + j.partials[k * kDiagSlots + s];
-    o[s] = v;
+    diag_final(j.partials, j.nblocks, j.status, out + (size_t)blockIdx.x * (kDiagSlots + 1));
 }
 
 // ------------------------------------------------------------------------
@@ -2272,11 +2371,8 @@ __global__ void __launch_bounds__(kStaticThreads) k_sums_static(const InstDesc* 
         const int y = (int)(t / D->nx), x = (int)(t % D->nx);
         R v[18];
         load18(buf, D->plane, (long long)y * D->pitch + x, v);
-        double w[18];
-#pragma unroll
-        for (int q = 0; q < 18; ++q) w[q] = (double)v[q];
         double rd, jx, jy, sg;
-        lbm::node_sums(w, w + 9, rd, jx, jy, sg);
+        node_sums_fp64(v, rd, jx, jy, sg);
         acc[0] += rd;
         acc[1] += jx;
         acc[2] += jy;
@@ -3025,6 +3121,11 @@ int grid_for(long long nn) {
     return (int)std::max<long long>(1, std::min<long long>(g, 152 * 8));
 }
 
+// One node per thread up to 16 CTAs per SM.
+int macro_grid(long long nn) {
+    return (int)std::max<long long>(1, std::min<long long>((nn + kMacroThreads - 1) / kMacroThreads, 152 * 16));
+}
+
 lbm_status check_launch() {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(LBM_ECUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
@@ -3495,8 +3596,8 @@ lbm_status lbm_sync(lbm_ctx* c) {
 lbm_status lbm_macros_device(lbm_ctx* c, double* rho, double* ux, double* uy, double* T, double* p) {
     if (!c || !c->eos_set) return fail(LBM_EINVAL, "context not initialised");
     const long long nn = (long long)c->cfg.nx * c->cfg.ny;
-    if (is_fp32(c)) k_macros<float><<<grid_for(nn), 256, 0, c->stream>>>(c->d_desc, cur_buf(c), rho, ux, uy, T, p);
-    else k_macros<double><<<grid_for(nn), 256, 0, c->stream>>>(c->d_desc, cur_buf(c), rho, ux, uy, T, p);
+    if (is_fp32(c)) k_macros<float><<<macro_grid(nn), kMacroThreads, 0, c->stream>>>(c->d_desc, cur_buf(c), rho, ux, uy, T, p);
+    else k_macros<double><<<macro_grid(nn), kMacroThreads, 0, c->stream>>>(c->d_desc, cur_buf(c), rho, ux, uy, T, p);
     return check_launch();
 }
 
@@ -3601,7 +3702,9 @@ static lbm_status diag_outputs(lbm_ctx* c, const double* acc, int snapshot, int 
     const Params<double>& P = c->h.pd;
     out8[0] = nn * P.rho0 + acc[0];
     out8[1] = nn * P.rho0 * P.E0 + acc[1];
-    out8[2] = acc[2];
+    const double Lx = c->h.px ? c->cfg.nx : c->cfg.nx - 1, Ly = c->h.py ? c->cfg.ny : c->cfg.ny - 1;
+    // the weights of the trapezoid rule add up to Lx Ly
+    out8[2] = 1.0 + acc[2] / (P.p0 * Lx * Ly);
     double r = 0.0;
     if (have) {
         const double ru = acc[4] > 0 ? std::sqrt(acc[3] / acc[4]) : 0.0;
@@ -3610,8 +3713,8 @@ static lbm_status diag_outputs(lbm_ctx* c, const double* acc, int snapshot, int 
     }
     out8[3] = r;
     out8[4] = acc[7];
-    out8[5] = acc[8];
-    out8[6] = acc[9] / nn;
+    out8[5] = std::sqrt(acc[8]);
+    out8[6] = P.T0 + acc[9] / nn;
     out8[7] = (double)c->steps;
     if (snapshot) c->have_snap = true;
     if (acc[7] > 0) {
@@ -3623,20 +3726,20 @@ static lbm_status diag_outputs(lbm_ctx* c, const double* acc, int snapshot, int 
 
 lbm_status lbm_diagnostics(lbm_ctx* c, int snapshot, double* out8) {
     if (!c || !c->eos_set || !out8) return fail(LBM_EINVAL, "bad arguments");
-    const int have = c->have_snap ? 1 : 0;
+    const int have = c->have_snap ? 1 : 0, nblocks = diag_blocks((long long)c->cfg.nx * c->cfg.ny);
     if (is_fp32(c))
-        k_diag<float><<<kDiagBlocks, kDiagThreads, 0, c->stream>>>(c->d_desc, cur_buf(c), c->d_snap, snapshot, have, c->d_partials);
+        k_diag<float><<<nblocks, kDiagThreads, 0, c->stream>>>(c->d_desc, cur_buf(c), c->d_snap, snapshot, have, c->d_partials);
     else
-        k_diag<double><<<kDiagBlocks, kDiagThreads, 0, c->stream>>>(c->d_desc, cur_buf(c), c->d_snap, snapshot, have, c->d_partials);
-    k_diag_final<<<1, 32, 0, c->stream>>>(c->d_partials, kDiagBlocks, c->d_diag);
+        k_diag<double><<<nblocks, kDiagThreads, 0, c->stream>>>(c->d_desc, cur_buf(c), c->d_snap, snapshot, have, c->d_partials);
+    k_diag_final<<<1, 32 * kDiagSlots, 0, c->stream>>>(c->d_partials, nblocks, c->d_status, c->d_diag);
     lbm_status st = check_launch();
     if (st != LBM_OK) return st;
-    double acc[kDiagSlots];
+    double acc[kDiagSlots + 1];
     CUDA_TRY(cudaMemcpyAsync(acc, c->d_diag, sizeof(acc), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     st = diag_outputs(c, acc, snapshot, have, out8);
     if (st != LBM_OK) return st;
-    return read_status(c);
+    return status_bits(c, (unsigned int)acc[kDiagSlots]);
 }
 
 // ------------------------------------------------------------------------
@@ -4013,18 +4116,19 @@ lbm_status lbm_batch_diagnostics(lbm_batch* b, int snapshot, double* out8n, int*
     }
     std::vector<DiagJob> jobs(n);
     std::vector<int> have(n);
-    int n32 = 0;
+    int n32 = 0, blocks[2] = {0, 0};  // of the FP64 and of the FP32 members
     for (int k = 0; k < n; ++k) {
         lbm_ctx* c = b->ctxs[b->diag_order[k]];
+        const int pr = is_fp32(c) ? 1 : 0, nblocks = diag_blocks((long long)c->cfg.nx * c->cfg.ny);
         have[k] = c->have_snap ? 1 : 0;
-        jobs[k] = DiagJob{c->d_desc, c->d_snap, c->d_partials, c->d_status, cur_buf(c), have[k]};
-        n32 += is_fp32(c) ? 1 : 0;
+        jobs[k] = DiagJob{c->d_desc, c->d_snap, c->d_partials, c->d_status, cur_buf(c), have[k], blocks[pr], nblocks};
+        blocks[pr] += nblocks;
+        n32 += pr;
     }
     CUDA_TRY(cudaMemcpyAsync(b->d_jobs, jobs.data(), n * sizeof(DiagJob), cudaMemcpyHostToDevice, b->stream));
-    if (n32) k_diag_batch<float><<<dim3(kDiagBlocks, n32), kDiagThreads, 0, b->stream>>>(b->d_jobs, snapshot);
-    if (n > n32)
-        k_diag_batch<double><<<dim3(kDiagBlocks, n - n32), kDiagThreads, 0, b->stream>>>(b->d_jobs + n32, snapshot);
-    k_diag_final_batch<<<n, 32, 0, b->stream>>>(b->d_jobs, kDiagBlocks, b->d_diag_out);
+    if (n32) k_diag_batch<float><<<blocks[1], kDiagThreads, 0, b->stream>>>(b->d_jobs, n32, snapshot);
+    if (n > n32) k_diag_batch<double><<<blocks[0], kDiagThreads, 0, b->stream>>>(b->d_jobs + n32, n - n32, snapshot);
+    k_diag_final_batch<<<n, 32 * kDiagSlots, 0, b->stream>>>(b->d_jobs, b->d_diag_out);
     lbm_status st = check_launch();
     if (st != LBM_OK) return st;
     std::vector<double> acc((size_t)n * (kDiagSlots + 1));
@@ -4092,8 +4196,8 @@ lbm_status lbm_batch_macros(lbm_batch* b, double* const* rho, double* const* ux,
             host[k] = fields[k] ? fields[k][i] : nullptr;
             dev[k] = host[k] ? c->d_stage + k * nn : nullptr;
         }
-        if (is_fp32(c)) k_macros<float><<<grid_for(nn), 256, 0, b->stream>>>(c->d_desc, cur_buf(c), dev[0], dev[1], dev[2], dev[3], dev[4]);
-        else k_macros<double><<<grid_for(nn), 256, 0, b->stream>>>(c->d_desc, cur_buf(c), dev[0], dev[1], dev[2], dev[3], dev[4]);
+        if (is_fp32(c)) k_macros<float><<<macro_grid(nn), kMacroThreads, 0, b->stream>>>(c->d_desc, cur_buf(c), dev[0], dev[1], dev[2], dev[3], dev[4]);
+        else k_macros<double><<<macro_grid(nn), kMacroThreads, 0, b->stream>>>(c->d_desc, cur_buf(c), dev[0], dev[1], dev[2], dev[3], dev[4]);
         lbm_status st = check_launch();
         if (st != LBM_OK) return st;
         for (int k = 0; k < 5; ++k)
