@@ -1765,25 +1765,37 @@ struct Field {
 };
 constexpr int kNodeThreads = 128;
 
+__host__ __device__ inline int node_ctas(long long n, int per_cta = kNodeThreads) { return (int)((n + per_cta - 1) / per_cta); }
+__device__ __forceinline__ NWork node_item(int block, long long n0, long long end, int per_cta, int kind) {
+    const long long first = n0 + (long long)block * per_cta;
+    return NWork{0, (int)first, (int)min((long long)per_cta, end - first), kind, 0, 0};
+}
+// The CTA's work: an entry of a batch's table, or (work null) its share of
+// the lone lattice descs[0], per_cta nodes a CTA.  k_collide_node and
+// k_collide_node2: every node or pair of nodes.  k_prep: the wall nodes,
+// whose work is longest, and then the rows that hold other nodes.
+__device__ __forceinline__ NWork collide_work(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta,
+                                              bool pairs) {
+    if (work) return work[blockIdx.x];
+    const InstDesc* D = descs[0];
+    return node_item(blockIdx.x, 0, (long long)(pairs ? (D->nx + 1) >> 1 : D->nx) * D->ny, per_cta, kInnerNodes);
+}
+__device__ __forceinline__ NWork prep_work(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta) {
+    if (work) return work[blockIdx.x];
+    const InstDesc* D = descs[0];
+    const int nwall = wall_count(D->nx, D->ny, D->px, D->py), wall_ctas = node_ctas(nwall), edge = D->py ? 0 : 1;
+    if ((int)blockIdx.x < wall_ctas) return node_item(blockIdx.x, 0, nwall, kNodeThreads, kWallNodes);
+    return node_item(blockIdx.x - wall_ctas, (long long)D->nx * edge, (long long)D->nx * (D->ny - edge), per_cta, kInnerNodes);
+}
+
 // wall_mode 0: macros of every node of the current buffer, as it stands
 // (first launch of a stepping call).  wall_mode 1: after a step, on the
 // buffer that it pushed into.
 template <typename R>
-__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 4 : 2)
-    k_prep(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int step_par, int wall_mode,
-           long long* counter) {
-    __shared__ Params<R> P;
-    const NWork w = work[blockIdx.x];
-    const InstDesc* D = descs[w.inst];
-    load_params(&P, &dparams<R>(D));
-    __syncthreads();
-    wait_for_previous();
-    if (counter && blockIdx.x == 0 && threadIdx.x == 0) *counter += 1;
-    if ((int)threadIdx.x >= w.cnt) return;
+__device__ __forceinline__ void prep_node(const NWork& w, const InstDesc* D, const Params<R>& P, R* buf, int wall_mode, int i) {
     const int nx = D->nx, ny = D->ny, pitch = D->pitch;
     const long long plane = D->plane;
-    R* buf = reinterpret_cast<R*>(D->buf[w.par ^ step_par ^ wall_mode]);
-    const int k = w.n0 + threadIdx.x;
+    const int k = w.n0 + i;
     int x, y;
     R v[18];
     if (w.kind == kWallNodes) {
@@ -1807,7 +1819,7 @@ __global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 4 : 2)
     }
     Mac<R> m;
     node_macros(P, v, m);
-    let_next_start();
+    if (i + kNodeThreads >= w.cnt) let_next_start();
     const Field<R> F(D->field, (long long)nx * ny);
     const int t = y * nx + x;
     F.rp[t] = RhoP<R>{m.rho_d, m.p_d};
@@ -1818,14 +1830,32 @@ __global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 4 : 2)
     }
 }
 
+// Five CTAs per SM in FP32 (102 registers): 64 small lattices take 29.2 us
+// per step against 32.7 us with four, 768^2 30.2 against 33.0.
+template <typename R>
+__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 5 : 2)
+    k_prep(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta, int step_par, int wall_mode,
+           long long* counter) {
+    __shared__ Params<R> P;
+    const NWork w = prep_work(work, descs, per_cta);
+    const InstDesc* D = descs[w.inst];
+    load_params(&P, &dparams<R>(D));
+    __syncthreads();
+    wait_for_previous();
+    if (counter && blockIdx.x == 0 && threadIdx.x == 0) *counter += 1;
+    R* buf = reinterpret_cast<R*>(D->buf[w.par ^ step_par ^ wall_mode]);
+    for (int i = threadIdx.x; i < w.cnt; i += kNodeThreads) prep_node(w, D, P, buf, wall_mode, i);
+}
+
 template <typename R, int MC>
-__device__ __forceinline__ void collide_node(const NWork& w, const InstDesc* D, const Params<R>& P, int step_par, uint32_t step_hash) {
+__device__ __forceinline__ void collide_node(const NWork& w, const InstDesc* D, const Params<R>& P, int step_par, uint32_t step_hash,
+                                             int i) {
     const int nx = D->nx, ny = D->ny, pitch = D->pitch, px = D->px, py = D->py;
     const long long plane = D->plane;
     const int b = w.par ^ step_par;
     const R* src = reinterpret_cast<const R*>(D->buf[b]);
     R* __restrict__ dst = reinterpret_cast<R*>(D->buf[b ^ 1]);
-    const int t = w.n0 + threadIdx.x;
+    const int t = w.n0 + i;
     const int y = t / nx, x = t - y * nx;
     R v[18];
     load18<R>(src, plane, (long long)y * pitch + x, v);
@@ -1887,24 +1917,25 @@ __device__ __forceinline__ void collide_node(const NWork& w, const InstDesc* D, 
     if (!(lbm::finite(m.rho_d) && lbm::finite(m.T_d))) atomicOr(D->status, 1u);
     AddDither add(mix32(step_hash ^ ((uint32_t)y * 0x85ebca77u + (uint32_t)x * 0xc2b2ae3du)), (float)P.dither);
     lbm::collide<MC>(P, m, v, v + 9, grx, gry, gpx, gpy, add);
-    let_next_start();
+    if (i + kNodeThreads >= w.cnt) let_next_start();
     push_node(dst, v, x, y, nx, ny, pitch, plane, px, py);
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 4 : 2)
-    k_collide_node(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int step_par,
+__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 5 : 2)
+    k_collide_node(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta, int step_par,
                    const long long* counter) {
     __shared__ Params<R> P;
-    const NWork w = work[blockIdx.x];
+    const NWork w = collide_work(work, descs, per_cta, false);
     const InstDesc* D = descs[w.inst];
     load_params(&P, &dparams<R>(D));
     __syncthreads();
     wait_for_previous();
     const uint32_t step_hash = mix32((uint32_t)(w.step0 + *counter) * 0x9e3779b1u + 0x632be5abu);
-    if ((int)threadIdx.x >= w.cnt) return;
-    if (D->mc == lbm::MODEL_CAVITY) collide_node<R, lbm::MODEL_CAVITY>(w, D, P, step_par, step_hash);
-    else collide_node<R, lbm::MODEL_ANY>(w, D, P, step_par, step_hash);
+    for (int i = threadIdx.x; i < w.cnt; i += kNodeThreads) {
+        if (D->mc == lbm::MODEL_CAVITY) collide_node<R, lbm::MODEL_CAVITY>(w, D, P, step_par, step_hash, i);
+        else collide_node<R, lbm::MODEL_ANY>(w, D, P, step_par, step_hash, i);
+    }
 }
 
 // k_collide_node for two neighbouring nodes per thread in packed FP32: the
@@ -1912,13 +1943,13 @@ __global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 4 : 2)
 // strips those are.
 template <int MC>
 __device__ __forceinline__ void collide_node2(const NWork& w, const InstDesc* D, const Params<f2>& P, float dscale, int step_par,
-                                              uint32_t step_hash) {
+                                              uint32_t step_hash, int i) {
     const int nx = D->nx, ny = D->ny, pitch = D->pitch, px = D->px, py = D->py;
     const long long plane = D->plane;
     const int b = w.par ^ step_par;
     const float* src = reinterpret_cast<const float*>(D->buf[b]);
     float* __restrict__ dst = reinterpret_cast<float*>(D->buf[b ^ 1]);
-    const int per_row = (nx + 1) >> 1, t2 = w.n0 + threadIdx.x;
+    const int per_row = (nx + 1) >> 1, t2 = w.n0 + i;
     const int y = t2 / per_row, xa = 2 * (t2 - y * per_row), xb = xa + 1;
     const bool act_b = xb < nx;
     f2 v[18];
@@ -1988,15 +2019,15 @@ __device__ __forceinline__ void collide_node2(const NWork& w, const InstDesc* D,
         atomicOr(D->status, 1u);
     AddDither2 add(mix32(step_hash ^ ((uint32_t)y * 0x85ebca77u + (uint32_t)xa * 0xc2b2ae3du)), dscale);
     lbm::collide<MC>(P, mf, v, v + 9, grx, gry, gpx, gpy, add);
-    let_next_start();
+    if (i + kNodeThreads >= w.cnt) let_next_start();
     push_pair(dst, v, xa, act_b, y, nx, ny, pitch, plane, px, py);
 }
 
 __global__ void __launch_bounds__(kNodeThreads, 3)
-    k_collide_node2(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int step_par,
+    k_collide_node2(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta, int step_par,
                     const long long* counter) {
     __shared__ Params<f2> P;
-    const NWork w = work[blockIdx.x];
+    const NWork w = collide_work(work, descs, per_cta, true);
     const InstDesc* D = descs[w.inst];
     // Params<f2> holds each number of Params<float> twice, then the same four integers
     constexpr int nf = offsetof(Params<float>, eos) / sizeof(float);
@@ -2007,9 +2038,10 @@ __global__ void __launch_bounds__(kNodeThreads, 3)
     __syncthreads();
     wait_for_previous();
     const uint32_t step_hash = mix32((uint32_t)(w.step0 + *counter) * 0x9e3779b1u + 0x632be5abu);
-    if ((int)threadIdx.x >= w.cnt) return;
-    if (D->mc == lbm::MODEL_CAVITY) collide_node2<lbm::MODEL_CAVITY>(w, D, P, D->pf.dither, step_par, step_hash);
-    else collide_node2<lbm::MODEL_ANY>(w, D, P, D->pf.dither, step_par, step_hash);
+    for (int i = threadIdx.x; i < w.cnt; i += kNodeThreads) {
+        if (D->mc == lbm::MODEL_CAVITY) collide_node2<lbm::MODEL_CAVITY>(w, D, P, D->pf.dither, step_par, step_hash, i);
+        else collide_node2<lbm::MODEL_ANY>(w, D, P, D->pf.dither, step_par, step_hash, i);
+    }
 }
 
 // ------------------------------------------------------------------------
@@ -2600,8 +2632,8 @@ struct lbm_ctx {
     int device = 0;         // device current at lbm_create, which holds the workspace
     BWork* d_bwork = nullptr;
     int n_bwork = 0;
-    NWork* d_nwork = nullptr;  // node kernels: n_node items of k_collide_node, then n_prep of k_prep
-    int n_node = 0, n_prep = 0;
+    int n_node = 0, n_prep = 0;  // CTAs of the node kernels, 0 when the lone lattice steps through strips
+    int node_per_cta = 0, prep_per_cta = 0;
     long steps = 0;
     bool eos_set = false, have_snap = false;
     lbm_status sticky = LBM_OK;
@@ -2609,7 +2641,6 @@ struct lbm_ctx {
     double f_rest[9] = {0}, g_rest[9] = {0};
     std::vector<Work> h_work;
     std::vector<BWork> h_bwork;
-    std::vector<NWork> h_nwork;
 };
 
 // Fused-kernel variants: strips of 32, 64, 128 columns, one node per thread
@@ -2747,25 +2778,39 @@ void ensure_tick(std::vector<BWork>& v, int inst, int par) {
     }
 }
 
+// Nodes (or pairs) per CTA of a node kernel: 128, and up to `most` times as
+// many where the launch would otherwise be more than one fill of the GPU, so
+// that a CTA's set-up (work item, descriptor, parameters) serves more nodes.
+// Two in FP32 (64 small lattices: 27.3 us per step against 29.2 us with one
+// and 29.0 us with four) but one for pairs, and four for k_prep in FP64, where
+// one tile is 51 instructions (298 us against 305 us), against one for the
+// collision, whose 320 want an even load (298 us against 316 us with two).
+int per_cta_for(long long nodes, int ctas_per_sm, int most) {
+    const long long tiles = nodes / ((long long)kNodeThreads * 152 * ctas_per_sm);
+    return kNodeThreads * (int)std::max<long long>(1, std::min<long long>(most, tiles));
+}
+
 // Work items of the node kernels for one lattice: every node for
 // k_collide_node; the wall nodes, whose work is longest, and then the rows
 // that hold other nodes for k_prep.
-void add_node_work(const lbm_config& c, int inst, int par, bool pairs, long long step0, std::vector<NWork>& v) {
+void add_node_work(const lbm_config& c, int inst, int par, bool pairs, long long step0, int per_cta, std::vector<NWork>& v) {
     const long long nn = (long long)(pairs ? (c.nx + 1) / 2 : c.nx) * c.ny;
-    for (long long n0 = 0; n0 < nn; n0 += kNodeThreads)
-        v.push_back(NWork{inst, (int)n0, (int)std::min<long long>(kNodeThreads, nn - n0), kInnerNodes, par, step0});
+    for (long long n0 = 0; n0 < nn; n0 += per_cta)
+        v.push_back(NWork{inst, (int)n0, (int)std::min<long long>(per_cta, nn - n0), kInnerNodes, par, step0});
 }
 void add_prep_wall(const lbm_config& c, int inst, int par, std::vector<NWork>& v) {
     const int n = wall_count(c.nx, c.ny, c.wall[LBM_WALL_W].periodic != 0, c.wall[LBM_WALL_S].periodic != 0);
     for (int n0 = 0; n0 < n; n0 += kNodeThreads)
         v.push_back(NWork{inst, n0, std::min(kNodeThreads, n - n0), kWallNodes, par, 0});
 }
-void add_prep_inner(const lbm_config& c, int inst, int par, std::vector<NWork>& v) {
+void add_prep_inner(const lbm_config& c, int inst, int par, int per_cta, std::vector<NWork>& v) {
     const int edge = c.wall[LBM_WALL_S].periodic ? 0 : 1;
     const long long hi = (long long)c.nx * (c.ny - edge);
-    for (long long n0 = (long long)c.nx * edge; n0 < hi; n0 += kNodeThreads)
-        v.push_back(NWork{inst, (int)n0, (int)std::min<long long>(kNodeThreads, hi - n0), kInnerNodes, par, 0});
+    for (long long n0 = (long long)c.nx * edge; n0 < hi; n0 += per_cta)
+        v.push_back(NWork{inst, (int)n0, (int)std::min<long long>(per_cta, hi - n0), kInnerNodes, par, 0});
 }
+
+bool is_fp32(const lbm_ctx* c) { return c->cfg.precision == LBM_FP32_DEV; }
 
 // Whether a lattice steps through the node kernels: always when lbm_set_tile
 // chose them; with a default shape, FP64 lattices always, and FP32 lattices
@@ -2778,6 +2823,10 @@ bool node_kernels(const lbm_ctx* c, long long nodes) {
 // Which of them: 0 FP64, 1 FP32, 2 FP32 in pairs (lattices whose strips are paired).
 enum { kNode64 = 0, kNode32 = 1, kNodePair = 2, kNodeKinds = 3 };
 int node_kind(const lbm_ctx* c) { return c->cfg.precision == LBM_FP64 ? kNode64 : c->pair == 1 ? kNodePair : kNode32; }
+int collide_per_cta(int kind, long long nodes) {
+    return kind == kNode32 ? per_cta_for(nodes, 5, 2) : kNodeThreads;
+}
+int prep_per_cta(bool fp32, long long nodes) { return fp32 ? per_cta_for(nodes, 5, 2) : per_cta_for(nodes, 2, 4); }
 
 // Default launch shape.  Lattices up to 160 columns wide take warp strips
 // of 30 columns (pair 4, same bits as pair 0): they waste fewer lanes there
@@ -2870,22 +2919,17 @@ lbm_status encode_windows(lbm_ctx* c) {
 
 long long resident_ctas(int vi, bool fp32);
 int variant_index(int bx, int pair);
-bool is_fp32(const lbm_ctx* c);
 
 lbm_status upload_work(lbm_ctx* c) {
     if (c->d_work) { cudaFree(c->d_work); c->d_work = nullptr; }
-    if (c->d_nwork) { cudaFree(c->d_nwork); c->d_nwork = nullptr; }
     c->n_node = c->n_prep = 0;
     if (node_kernels(c, (long long)c->cfg.nx * c->cfg.ny)) {
-        std::vector<NWork>& v = c->h_nwork;
-        v.clear();
-        add_node_work(c->cfg, 0, 0, node_kind(c) == kNodePair, 0, v);
-        c->n_node = (int)v.size();
-        add_prep_wall(c->cfg, 0, 0, v);
-        add_prep_inner(c->cfg, 0, 0, v);
-        c->n_prep = (int)v.size() - c->n_node;
-        CUDA_TRY(cudaMalloc(&c->d_nwork, v.size() * sizeof(NWork)));
-        CUDA_TRY(cudaMemcpyAsync(c->d_nwork, v.data(), v.size() * sizeof(NWork), cudaMemcpyHostToDevice, c->stream));
+        // no table: the kernels find a lone lattice's work by themselves
+        const int nx = c->cfg.nx, ny = c->cfg.ny, edge = c->h.py ? 0 : 1;
+        c->node_per_cta = collide_per_cta(node_kind(c), (long long)nx * ny);
+        c->prep_per_cta = prep_per_cta(is_fp32(c), (long long)nx * ny);
+        c->n_node = node_ctas((long long)(node_kind(c) == kNodePair ? (nx + 1) / 2 : nx) * ny, c->node_per_cta);
+        c->n_prep = node_ctas(wall_count(nx, ny, c->h.px, c->h.py)) + node_ctas((long long)nx * (ny - 2 * edge), c->prep_per_cta);
         return LBM_OK;
     }
     c->h_work = make_work(c->cfg, 0, c->bx, c->by, 0, 0);
@@ -3165,17 +3209,17 @@ void launch_boundary(const BWork* work, int n, InstDesc* const* descs, int par, 
     launch_step(k_boundary<R>, n, 128, 0, s, work, descs, par, counter);
 }
 
-void launch_node(int kind, const NWork* work, int n, InstDesc* const* descs, int par, const long long* counter, cudaStream_t s) {
+void launch_node(int kind, const NWork* work, int n, int per_cta, InstDesc* const* descs, int par, const long long* counter, cudaStream_t s) {
     if (n <= 0) return;
-    if (kind == kNodePair) launch_step(k_collide_node2, n, kNodeThreads, 0, s, work, descs, par, counter);
-    else if (kind == kNode32) launch_step(k_collide_node<float>, n, kNodeThreads, 0, s, work, descs, par, counter);
-    else launch_step(k_collide_node<double>, n, kNodeThreads, 0, s, work, descs, par, counter);
+    if (kind == kNodePair) launch_step(k_collide_node2, n, kNodeThreads, 0, s, work, descs, per_cta, par, counter);
+    else if (kind == kNode32) launch_step(k_collide_node<float>, n, kNodeThreads, 0, s, work, descs, per_cta, par, counter);
+    else launch_step(k_collide_node<double>, n, kNodeThreads, 0, s, work, descs, per_cta, par, counter);
 }
-void launch_prep(bool fp32, const NWork* work, int n, InstDesc* const* descs, int par, int wall_mode, long long* counter,
+void launch_prep(bool fp32, const NWork* work, int n, int per_cta, InstDesc* const* descs, int par, int wall_mode, long long* counter,
                  cudaStream_t s) {
     if (n <= 0) return;
-    if (fp32) launch_step(k_prep<float>, n, kNodeThreads, 0, s, work, descs, par, wall_mode, counter);
-    else launch_step(k_prep<double>, n, kNodeThreads, 0, s, work, descs, par, wall_mode, counter);
+    if (fp32) launch_step(k_prep<float>, n, kNodeThreads, 0, s, work, descs, per_cta, par, wall_mode, counter);
+    else launch_step(k_prep<double>, n, kNodeThreads, 0, s, work, descs, per_cta, par, wall_mode, counter);
 }
 
 int grid_for(long long nn) {
@@ -3217,7 +3261,6 @@ lbm_status read_status(lbm_ctx* c) {
     return status_bits(c, st);
 }
 
-bool is_fp32(const lbm_ctx* c) { return c->cfg.precision == LBM_FP32_DEV; }
 
 int cur_buf(const lbm_ctx* c) { return (int)(c->steps & 1); }
 
@@ -3306,8 +3349,7 @@ lbm_status lbm_create(const lbm_config* cfg, void* workspace, size_t workspace_b
     if (cudaMemcpyAsync(c->d_descs, &p, sizeof(p), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
         return cleanup(fail(LBM_ECUDA, "descs upload"));
     default_shape(*cfg, lbm::MODEL_ANY, c->bx, c->pair);
-    c->by = default_rows(*cfg, c->pair);
-    if ((st = upload_work(c)) != LBM_OK) return cleanup(st);
+    c->by = default_rows(*cfg, c->pair);  // its table follows in lbm_set_eos
     c->h_bwork = make_bwork(*cfg, 0, 0);
     ensure_tick(c->h_bwork, 0, 0);
     c->n_bwork = (int)c->h_bwork.size();
@@ -3329,7 +3371,6 @@ lbm_status lbm_destroy(lbm_ctx* c) {
     else cudaDeviceSynchronize();
     if (c->d_work) cudaFree(c->d_work);
     if (c->d_bwork) cudaFree(c->d_bwork);
-    if (c->d_nwork) cudaFree(c->d_nwork);
     if (c->own_ws && c->ws) cudaFree(c->ws);
     delete c;
     return LBM_OK;
@@ -3438,7 +3479,7 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
         // the default shape depends on the model class
         int bx = 0, pair = 0;
         default_shape(k, c->mc, bx, pair);
-        if (bx != c->bx || pair != c->pair) {
+        if (bx != c->bx || pair != c->pair || !(c->d_work || c->n_node)) {
             c->bx = bx;
             c->pair = pair;
             c->by = default_rows(k, pair);
@@ -3629,13 +3670,12 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
     const long long base = c->steps;
     CUDA_TRY(cudaMemcpyAsync(c->d_counter, &base, sizeof(base), cudaMemcpyHostToDevice, c->stream));
     const bool f32 = is_fp32(c);
-    const NWork* prep = c->d_nwork + c->n_node;
-    launch_prep(f32, prep, c->n_prep, c->d_descs, cur_buf(c), 0, nullptr, c->stream);
+    launch_prep(f32, nullptr, c->n_prep, c->prep_per_cta, c->d_descs, cur_buf(c), 0, nullptr, c->stream);
     for (long s = 0; s < nsteps; ++s) {
         const int par = (int)((c->steps + s) & 1);
         if (c->n_node) {
-            launch_node(node_kind(c), c->d_nwork, c->n_node, c->d_descs, par, c->d_counter, c->stream);
-            launch_prep(f32, prep, c->n_prep, c->d_descs, par, 1, c->d_counter, c->stream);
+            launch_node(node_kind(c), nullptr, c->n_node, c->node_per_cta, c->d_descs, par, c->d_counter, c->stream);
+            launch_prep(f32, nullptr, c->n_prep, c->prep_per_cta, c->d_descs, par, 1, c->d_counter, c->stream);
         } else if (f32) {
             launch_collide<float>(c->d_work, c->n_work, variant_index(c->bx, c->pair), c->mc, c->d_descs, par, c->d_counter, c->stream);
             launch_boundary<float>(c->d_bwork, c->n_bwork, c->d_descs, par, c->d_counter, c->stream);
@@ -3863,12 +3903,12 @@ lbm_status lbm_conserved_sums_static(const lbm_ctx* c, double* out4) {
 // first step after this call reads.
 static void batch_launch_first(lbm_batch* b, const LaunchSet& ls, int par, cudaStream_t st) {
     for (int pr = 0; pr < 2; ++pr)
-        launch_prep(pr == 1, b->d_nwork + ls.p_off[pr], ls.p_cnt[pr], b->d_descs, par, 0, nullptr, st);
+        launch_prep(pr == 1, b->d_nwork + ls.p_off[pr], ls.p_cnt[pr], 0, b->d_descs, par, 0, nullptr, st);
 }
 
 static void batch_launch_collide(lbm_batch* b, const LaunchSet& ls, int par, cudaStream_t st) {
     for (int k = 0; k < kNodeKinds; ++k)
-        launch_node(k, b->d_nwork + ls.n_off[k], ls.n_cnt[k], b->d_descs, par, ls.counter, st);
+        launch_node(k, b->d_nwork + ls.n_off[k], ls.n_cnt[k], 0, b->d_descs, par, ls.counter, st);
     for (int pr = 0; pr < 2; ++pr)
         for (int vi = 0; vi < kVariants; ++vi)
             for (int mc = 0; mc < kModels; ++mc) {
@@ -3888,7 +3928,7 @@ static void batch_launch_boundary(lbm_batch* b, const LaunchSet& ls, int par, cu
     for (int k = 0; k < 4; ++k) {
         const int pr = k & 1;
         long long* ctr = k == last ? ls.counter : nullptr;
-        if (k >= 2) launch_prep(pr == 1, b->d_nwork + ls.p_off[pr], ls.p_cnt[pr], b->d_descs, par, 1, ctr, st);
+        if (k >= 2) launch_prep(pr == 1, b->d_nwork + ls.p_off[pr], ls.p_cnt[pr], 0, b->d_descs, par, 1, ctr, st);
         else if (pr) launch_boundary<float>(b->d_bwork + ls.b_off[pr], ls.b_cnt[pr], b->d_descs, par, ctr, st);
         else launch_boundary<double>(b->d_bwork + ls.b_off[pr], ls.b_cnt[pr], b->d_descs, par, ctr, st);
     }
@@ -3915,17 +3955,22 @@ static void build_launch_set(lbm_ctx* const* ctxs, const std::vector<int>& membe
         for (int i : members)
             if (node[i] && take(ctxs[i])) f(i, ctxs[i], (int)(ctxs[i]->steps & 1));
     };
+    long long nodes[kNodeKinds] = {0, 0, 0};
+    for (int i : members)
+        if (node[i]) nodes[node_kind(ctxs[i])] += (long long)ctxs[i]->cfg.nx * ctxs[i]->cfg.ny;
     for (int k = 0; k < kNodeKinds; ++k) {
+        const int per = collide_per_cta(k, nodes[k]);
         ls.n_off[k] = (int)nall.size();
         each([&](const lbm_ctx* c) { return node_kind(c) == k; },
-             [&](int i, const lbm_ctx* c, int par) { add_node_work(c->cfg, i, par, k == kNodePair, c->steps, nall); });
+             [&](int i, const lbm_ctx* c, int par) { add_node_work(c->cfg, i, par, k == kNodePair, c->steps, per, nall); });
         ls.n_cnt[k] = (int)nall.size() - ls.n_off[k];
     }
     for (int pr = 0; pr < 2; ++pr) {
         auto mine = [&](const lbm_ctx* c) { return is_fp32(c) == (pr == 1); };
+        const int per = prep_per_cta(pr == 1, pr ? nodes[kNode32] + nodes[kNodePair] : nodes[kNode64]);
         ls.p_off[pr] = (int)nall.size();
         each(mine, [&](int i, const lbm_ctx* c, int par) { add_prep_wall(c->cfg, i, par, nall); });
-        each(mine, [&](int i, const lbm_ctx* c, int par) { add_prep_inner(c->cfg, i, par, nall); });
+        each(mine, [&](int i, const lbm_ctx* c, int par) { add_prep_inner(c->cfg, i, par, per, nall); });
         ls.p_cnt[pr] = (int)nall.size() - ls.p_off[pr];
     }
     std::vector<Work> groups[2][kVariants][kModels];

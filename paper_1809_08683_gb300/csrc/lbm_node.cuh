@@ -723,14 +723,15 @@ LBM_HD void equilibrium(const Params<R>& P, const Mac<R>& mb, R* f, R* g) {
     inverse_moments(n, g);
 }
 
-// Sums over the 9 populations of a node: rho', j, sum g'.
+// Sums over the 9 populations of a node: rho', j, sum g'.  Added in the order
+// of moments(), so that a kernel that calls both adds once.
 template <typename R>
 LBM_HD void node_sums(const R* f, const R* g, R& rd, R& jx, R& jy, R& sg) {
-    rd = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
     const R d1 = f[5] - f[7], d2 = f[6] - f[8];
+    rd = f[0] + (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
     jx = (f[1] - f[3]) + (d1 - d2);
     jy = (f[2] - f[4]) + (d1 + d2);
-    sg = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+    sg = g[0] + (((g[1] + g[3]) + (g[2] + g[4])) + ((g[5] + g[7]) + (g[6] + g[8])));
 }
 
 }  // namespace lbm
