@@ -43,10 +43,14 @@ __device__ __forceinline__ f2 fdiv(const f2& a, const f2& b) {
 __device__ __forceinline__ f2 recip(const f2& b) { return fdiv(f2(1.0f), b); }
 __device__ __forceinline__ f2 root(const f2& a) { return f2(make_float2(sqrtf(a.v.x), sqrtf(a.v.y))); }
 
-__device__ __forceinline__ f2 cs_dev(const f2& b, const f2& rho0, const f2& Rg, const f2& rho_d, const f2& T,
-                                     const f2& T_d) {
-    return f2(make_float2((float)cs_dev1(b.v.x, rho0.v.x, Rg.v.x, rho_d.v.x, T.v.x, T_d.v.x),
-                          (float)cs_dev1(b.v.y, rho0.v.y, Rg.v.y, rho_d.v.y, T.v.y, T_d.v.y)));
+__device__ __forceinline__ f2 cs_dev(const f2* c, const f2* lo, const f2& rho_d, const f2& T, const f2& T_d) {
+    float k[7], l[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        k[i] = c[i].v.x;
+        l[i] = lo[i].v.x;
+    }
+    return f2(make_float2(cs_dev(k, l, rho_d.v.x, T.v.x, T_d.v.x), cs_dev(k, l, rho_d.v.y, T.v.y, T_d.v.y)));
 }
 
 }  // namespace lbm

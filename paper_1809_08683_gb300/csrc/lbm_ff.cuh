@@ -3,7 +3,8 @@
 // 48 significant bits in FP32 instructions.  lbm_peak_rates measures its
 // multiply-add rate next to the FP64 and FP32 FMA rates, the figures that
 // decide whether FP64-accurate node arithmetic is cheaper in FP32 pairs than
-// on GB300's FP64 pipe.  The algorithms are the error-free transformations
+// on GB300's FP64 pipe; the Carnahan-Starling pressure of FP32 lattices is
+// formed in it.  The algorithms are the error-free transformations
 // of Knuth (two-sum), Dekker (fast two-sum) and the FMA-based exact
 // product, combined as in the double-double literature (Hida, Li and
 // Bailey): every operation is accurate to a few units in 2^-48 relative,

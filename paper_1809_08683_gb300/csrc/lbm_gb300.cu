@@ -38,7 +38,6 @@
 
 #include "../../include/lbm.h"
 #include "lbm_f2.cuh"
-#include "lbm_ff.cuh"
 #include "lbm_node.cuh"
 
 using lbm::f2;
@@ -989,6 +988,10 @@ __device__ void broadcast_params(const Params<float>& a, Params<f2>& b) {
     BP(kk); BP(hh); BP(bb); BP(bbm2); BP(omk); BP(k2h); BP(gamma1); BP(gamma2); BP(k11); BP(k17); BP(k18);
     BP(k71); BP(k77); BP(k81); BP(k88); BP(Fx); BP(Fy); BP(cs_b0); BP(dither);
 #undef BP
+    for (int i = 0; i < 7; ++i) {
+        b.cs[i] = f2(a.cs[i]);
+        b.cs_lo[i] = f2(a.cs_lo[i]);
+    }
     b.eos = a.eos;
     b.visc = a.visc;
     b.force_mode = a.force_mode;
@@ -2597,6 +2600,10 @@ void convert_params(const Params<A>& a, Params<B>& b) {
     CP(kk); CP(hh); CP(bb); CP(bbm2); CP(omk); CP(k2h); CP(gamma1); CP(gamma2); CP(k11); CP(k17); CP(k18);
     CP(k71); CP(k77); CP(k81); CP(k88); CP(Fx); CP(Fy); CP(cs_b0); CP(dither);
 #undef CP
+    for (int i = 0; i < 7; ++i) {
+        b.cs[i] = (B)a.cs[i];
+        b.cs_lo[i] = (B)(a.cs[i] - (A)b.cs[i]);
+    }
     b.eos = a.eos;
     b.visc = a.visc;
     b.force_mode = a.force_mode;
@@ -3463,6 +3470,7 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
     P.Fx = k.force[0];
     P.Fy = k.force[1];
     P.cs_b0 = 1.0 - b * r0;
+    if (kind == LBM_EOS_CS) lbm::cs_constants(b, r0, Rg, P.cs);
     P.dither = c->round_mode == LBM_ROUND_NEAREST ? 0.0 : 1.0;
     P.eos = kind;
     P.visc = k.visc_law;
