@@ -217,7 +217,7 @@ lbm_status lbm_set_tile(lbm_ctx* ctx, int bx, int by, int pair);
  * nx <= 160; paired block strips, pair = 1, bx = 128, for wider FP32
  * lattices of the heated-cavity model class (see lbm_batch_create); block
  * strips, pair = 0, bx = 128, otherwise.  by = ny / 128 between 1 and 24
- * (FP32) or 8 (FP64); 3 ny / 512 between 1 and 12 for pair = 1.  by is
+ * (FP32) or 8 (FP64); 3 ny / 512 between 1 and 32 for pair = 1.  by is
  * the run length when the lattice is stepped alone; a batch uses runs of
  * up to 24 (FP32; 32 for pair = 1) or 8 (FP64) rows for members whose
  * shape was not set, shortened until the batch fills the GPU.  In either

@@ -681,7 +681,7 @@ __global__ void __launch_bounds__(BX, KEEP ? FusedTraits<R, BX>::MINB : FusedTra
             for (int q = 0; q < 18; ++q) v[q] = st[q * W];
             Mac<R> mf;
             if (KEEP) {
-                lbm::expand<MC>(P, mc, mf);
+                lbm::expand<MC>(P, mc, lbm::sum9(v + 9), mf);
             } else {
                 node_macros<MC>(P, v, mf);
                 if (!(lbm::finite(mf.rho_d) && lbm::finite(mf.T_d))) atomicOr(status, 1u);
@@ -932,7 +932,7 @@ __global__ void __launch_bounds__(32 * NW, WarpTraits<R>::WARPS_PER_SM / NW)
             const int sc = (k + 1) % S;
             load_node(sc, v);
             Mac<R> mf;
-            lbm::expand<MC>(P, mc, mf);
+            lbm::expand<MC>(P, mc, lbm::sum9(v + 9), mf);
             AddDither add(mix32(step_hash ^ ((uint32_t)j * 0x85ebca77u + (uint32_t)x * 0xc2b2ae3du)), dscale);
             // the DFs are fetched again for the final update, so that they
             // need not occupy registers through the collision
@@ -986,7 +986,7 @@ __device__ void broadcast_params(const Params<float>& a, Params<f2>& b) {
     BP(rho0); BP(T0); BP(E0); BP(Cv); BP(inv_Cv); BP(Rg); BP(eos_a); BP(eos_b); BP(p0); BP(rho0E0_p0);
     BP(rho0Cp0); BP(mu0); BP(mu0S); BP(inv_T0); BP(visc_S); BP(lam_fac); BP(nu_e); BP(mu_j); BP(beta2);
     BP(kk); BP(hh); BP(bb); BP(bbm2); BP(omk); BP(k2h); BP(gamma1); BP(gamma2); BP(k11); BP(k17); BP(k18);
-    BP(k71); BP(k77); BP(k81); BP(k88); BP(Fx); BP(Fy); BP(cs_b0); BP(dither);
+    BP(k71); BP(k77); BP(k81); BP(k88); BP(Fx); BP(Fy); BP(Fxh); BP(Fyh); BP(cs_b0); BP(dither);
 #undef BP
     for (int i = 0; i < 7; ++i) {
         b.cs[i] = f2(a.cs[i]);
@@ -1048,7 +1048,10 @@ __global__ void __launch_bounds__(BX / 2, (KEEP ? LBM_PAIR_WARPS_PER_SM : 12) * 
         s_abort = 0;
     }
     const int nx = D->nx, ny = D->ny, pitch = D->pitch, px = D->px, py = D->py;
-    const long long plane = D->plane;
+    // 18 planes fit 32-bit offsets (checked at creation).  Every register
+    // counts: at 168 a spilled one is reloaded per row past the little L1 that
+    // the row stages leave (4096^2: 452 us per step with two spilled, 442 with one).
+    const int plane = (int)D->plane;
     const int b = w.par ^ step_par;
     const float* src = reinterpret_cast<const float*>(D->buf[b]);
     float* __restrict__ dst = reinterpret_cast<float*>(D->buf[b ^ 1]);
@@ -1256,7 +1259,7 @@ __global__ void __launch_bounds__(BX / 2, (KEEP ? LBM_PAIR_WARPS_PER_SM : 12) * 
             for (int q = 0; q < 18; ++q) v[q] = f2(*reinterpret_cast<const float2*>(st + q * W));
             Mac<f2> mf;
             if (KEEP) {
-                lbm::expand<MC>(P2, mc, mf);
+                lbm::expand<MC>(P2, mc, lbm::sum9(v + 9), mf);
             } else {
                 f2 rd, jx, jy, sg;
                 lbm::node_sums(v, v + 9, rd, jx, jy, sg);
@@ -1549,7 +1552,7 @@ __global__ void __launch_bounds__(32 * NW, LBM_WARP2_WARPS_PER_SM / NW)
             f2 v[18];
             load_pair((k + 1) % S, v);
             Mac<f2> mf;
-            expand(P2, mc, mf);
+            expand(P2, mc, lbm::sum9(v + 9), mf);
             AddDither2 add(mix32(step_hash ^ ((uint32_t)j * 0x85ebca77u + (uint32_t)xa * 0xc2b2ae3du)), dscale);
             auto reload = [&](f2* f, f2*) {
                 asm volatile("" ::: "memory");
@@ -1795,36 +1798,12 @@ __device__ __forceinline__ NWork prep_work(const NWork* __restrict__ work, InstD
 // (first launch of a stepping call).  wall_mode 1: after a step, on the
 // buffer that it pushed into.
 template <typename R>
-__device__ __forceinline__ void prep_node(const NWork& w, const InstDesc* D, const Params<R>& P, R* buf, int wall_mode, int i) {
-    const int nx = D->nx, ny = D->ny, pitch = D->pitch;
-    const long long plane = D->plane;
-    const int k = w.n0 + i;
-    int x, y;
-    R v[18];
-    if (w.kind == kWallNodes) {
-        WallNode n;
-        wall_node(D, k, n);
-        x = n.x;
-        y = n.y;
-        if (wall_mode) {
-            rebuilt_wall_node(P, buf, plane, pitch, n, v);
-            store18<R>(buf, plane, (long long)y * pitch + x, v);
-        }
-    } else {
-        y = k / nx;
-        x = k - y * nx;
-        if ((!D->px && (x == 0 || x == nx - 1)) || (!D->py && (y == 0 || y == ny - 1))) return;
-    }
-    if (!(w.kind == kWallNodes && wall_mode)) {
-        const R* a = buf + (long long)y * pitch + x;
-#pragma unroll
-        for (int q = 0; q < 18; ++q) v[q] = a[q * plane];
-    }
+__device__ __forceinline__ void put_macros(const InstDesc* D, const Params<R>& P, const R* v, int x, int y, bool last) {
     Mac<R> m;
     node_macros(P, v, m);
-    if (i + kNodeThreads >= w.cnt) let_next_start();
-    const Field<R> F(D->field, (long long)nx * ny);
-    const int t = y * nx + x;
+    if (last) let_next_start();
+    const Field<R> F(D->field, (long long)D->nx * D->ny);
+    const int t = y * D->nx + x;
     F.rp[t] = RhoP<R>{m.rho_d, m.p_d};
     if (sizeof(R) == 8) {
         F.ux[t] = m.ux;
@@ -1832,11 +1811,39 @@ __device__ __forceinline__ void prep_node(const NWork& w, const InstDesc* D, con
         F.T[t] = m.T_d;
     }
 }
-
-// Five CTAs per SM in FP32 (102 registers): 64 small lattices take 29.2 us
-// per step against 32.7 us with four, 768^2 30.2 against 33.0.
 template <typename R>
-__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 5 : 2)
+__device__ __forceinline__ void prep_inner(const NWork& w, const InstDesc* D, const Params<R>& P, const R* buf, int i) {
+    const int nx = D->nx, ny = D->ny, k = w.n0 + i, y = k / nx, x = k - y * nx;
+    if ((!D->px && (x == 0 || x == nx - 1)) || (!D->py && (y == 0 || y == ny - 1))) return;
+    R v[18];
+    load18(buf, D->plane, (long long)y * D->pitch + x, v);
+    put_macros(D, P, v, x, y, i + kNodeThreads >= w.cnt);
+}
+template <typename R>
+__device__ __forceinline__ void prep_wall(const NWork& w, const InstDesc* D, const Params<R>& P, R* buf, int wall_mode, int i) {
+    const int pitch = D->pitch;
+    const long long plane = D->plane;
+    WallNode n;
+    wall_node(D, w.n0 + i, n);
+    const long long at = (long long)n.y * pitch + n.x;
+    R v[18];
+    if (wall_mode) {
+        rebuilt_wall_node(P, buf, plane, pitch, n, v);
+        store18<R>(buf, plane, at, v);
+    } else {
+        load18(buf, plane, at, v);
+    }
+    put_macros(D, P, v, n.x, n.y, true);
+}
+
+// Six CTAs per SM in FP32, at the price of a few spills on the wall path: 64
+// small lattices take 26.5 us per step against 27.6 us with four, 768^2 27.4
+// against 29.0; FP64 keeps its registers, whose spills would lengthen the
+// wall nodes' serial work (256^2: 74 us per step with two, 76 with three).
+// The two kinds of item share no code path: one common tail cost the inner
+// nodes their batched loads (64 small lattices 29.1 us).
+template <typename R>
+__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 6 : 2)
     k_prep(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta, int step_par, int wall_mode,
            long long* counter) {
     __shared__ Params<R> P;
@@ -1847,7 +1854,11 @@ __global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 5 : 2)
     wait_for_previous();
     if (counter && blockIdx.x == 0 && threadIdx.x == 0) *counter += 1;
     R* buf = reinterpret_cast<R*>(D->buf[w.par ^ step_par ^ wall_mode]);
-    for (int i = threadIdx.x; i < w.cnt; i += kNodeThreads) prep_node(w, D, P, buf, wall_mode, i);
+    if (w.kind == kWallNodes) {
+        if ((int)threadIdx.x < w.cnt) prep_wall(w, D, P, buf, wall_mode, threadIdx.x);
+    } else {
+        for (int i = threadIdx.x; i < w.cnt; i += kNodeThreads) prep_inner(w, D, P, buf, i);
+    }
 }
 
 template <typename R, int MC>
@@ -1908,12 +1919,7 @@ __device__ __forceinline__ void collide_node(const NWork& w, const InstDesc* D, 
         mk.uy = F.uy[t];
         mk.T_d = F.T[t];
         mk.p_d = c.p;
-        R rd, jx, jy, sg;
-        lbm::node_sums(v, v + 9, rd, jx, jy, sg);  // only sg is used
-        mk.rhoE_d = sg;
-        lbm::expand<MC>(P, mk, m);
-        m.rhoE_d = lbm::mad(R(0.5), m.qe, sg);
-        m.rhoH = P.rho0E0_p0 + m.rhoE_d + m.p_d;
+        lbm::expand<MC>(P, mk, lbm::sum9(v + 9), m);
     } else {
         node_macros<MC>(P, v, m);
     }
@@ -2598,7 +2604,7 @@ void convert_params(const Params<A>& a, Params<B>& b) {
     CP(rho0); CP(T0); CP(E0); CP(Cv); CP(inv_Cv); CP(Rg); CP(eos_a); CP(eos_b); CP(p0); CP(rho0E0_p0);
     CP(rho0Cp0); CP(mu0); CP(mu0S); CP(inv_T0); CP(visc_S); CP(lam_fac); CP(nu_e); CP(mu_j); CP(beta2);
     CP(kk); CP(hh); CP(bb); CP(bbm2); CP(omk); CP(k2h); CP(gamma1); CP(gamma2); CP(k11); CP(k17); CP(k18);
-    CP(k71); CP(k77); CP(k81); CP(k88); CP(Fx); CP(Fy); CP(cs_b0); CP(dither);
+    CP(k71); CP(k77); CP(k81); CP(k88); CP(Fx); CP(Fy); CP(Fxh); CP(Fyh); CP(cs_b0); CP(dither);
 #undef CP
     for (int i = 0; i < 7; ++i) {
         b.cs[i] = (B)a.cs[i];
@@ -2868,12 +2874,13 @@ long long cta_count(const lbm_config& c, int bx, int by) {
 // Rows per run for a lattice launched on its own.  Block and warp strips:
 // ny / 128, between 1 and the longest run (measured optimum on square FP32
 // lattices: 1-2 rows at 256^2, 4 at 512^2, 8 at 1024^2, 12-16 at 2048^2, 24
-// at 4096^2).  Paired block strips: 3 ny / 512, between 1 and 12 (measured:
-// 2-4 at 512^2, 6 at 1024^2, 8-12 at 2048^2, 12 at 4096^2).  A small
+// at 4096^2).  Paired block strips: 3 ny / 512, between 1 and 32 (measured:
+// 2-4 at 512^2, 6 at 1024^2, 8-12 at 2048^2; 4096^2: 442 us per step with 12
+// rows, 435 with 24, 433 with 32).  A small
 // lattice is latency-bound and gains more from spreading over more SMs than
 // it loses re-staging halo rows.
 int default_rows(const lbm_config& c, int pair) {
-    if (pair == 1) return std::max(1, std::min(std::min(batch_rows(c, pair), 12), c.ny * 3 / 512));
+    if (pair == 1) return std::max(1, std::min(batch_rows(c, pair), c.ny * 3 / 512));
     return std::max(1, std::min(batch_rows(c, pair), c.ny / 128));
 }
 
@@ -2915,7 +2922,7 @@ lbm_status encode_windows(lbm_ctx* c) {
         for (int b = 0; b < 2; ++b) {
             const CUresult r = enc(&c->h.tmap[k][b], f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64,
                                    3, c->h.buf[b], dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS)
                 return fail(LBM_ECUDA, "cuTensorMapEncodeTiled failed (code " + std::to_string((int)r) + ")");
@@ -3469,6 +3476,8 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
     P.k88 = 6.0 * P.bb * 2.0;
     P.Fx = k.force[0];
     P.Fy = k.force[1];
+    P.Fxh = 0.5 * P.Fx;
+    P.Fyh = 0.5 * P.Fy;
     P.cs_b0 = 1.0 - b * r0;
     if (kind == LBM_EOS_CS) lbm::cs_constants(b, r0, Rg, P.cs);
     P.dither = c->round_mode == LBM_ROUND_NEAREST ? 0.0 : 1.0;

@@ -130,7 +130,7 @@ struct Params {
     R beta2;          // -2 beta1 / (1 - varpi); alpha1 = -1, beta1 = 1, alpha2 = 1 are fixed
     R kk, hh, bb, bbm2, omk, k2h, gamma1, gamma2;  // bbm2 = -2 bb
     R k11, k17, k18, k71, k77, k81, k88;  // entries of R per 1/(1 + 6 nu) or 1/(1 + nu_e nu) (collide)
-    R Fx, Fy;
+    R Fx, Fy, Fxh, Fyh;  // force (or g) and half of it
     R cs_b0;  // 1 - b rho0 (cubic EOS)
     R cs[7], cs_lo[7];  // Carnahan-Starling constants (cs_constants) and, in FP32, what R leaves of them
     R dither; // FP32 storage: 1 rounds the stored deviations stochastically, 0 to nearest
@@ -162,11 +162,11 @@ struct Mac {
 
 // The part of Mac that the fused kernels keep in registers from a row's
 // macro pass to its collision; expand() rebuilds the rest with the same
-// operations as macros(), so an expanded state equals the original bit
-// for bit.
+// operations as macros() from it and sum g' (which the collision's moments
+// form anyway), so an expanded state equals the original bit for bit.
 template <typename R>
 struct MacC {
-    R rho_d, ir, ux, uy, rhoE_d, T_d, p_d;
+    R rho_d, ir, ux, uy, T_d, p_d;
 };
 
 // Carnahan-Starling deviation p - p0 with p = Z(e) rho R T, e = b rho / 4
@@ -265,12 +265,20 @@ LBM_HD void macros(const Params<R>& P, R rho_d, R jx, R jy, R sg, Mac<R>& m) {
     m.rho = P.rho0 + rho_d;
     m.ir = recip(m.rho);
     mac_force<MC>(P, m);
-    m.ux = MC == MODEL_CAVITY ? jx * m.ir : mad(R(0.5), m.Fx, jx) * m.ir;
-    m.uy = mad(R(0.5), m.Fy, jy) * m.ir;
+    // u = j / rho + a with a = F / (2 rho), and since q / (2 rho) = u . a,
+    // Cv T' = (sum g' - rho' E0) / rho + u . (a - u/2); q itself only enters
+    // the collision
+    R ax = P.Fxh, ay = P.Fyh;
+    if (!force_is_rho_g<MC>(P)) {
+        ax = ax * m.ir;
+        ay = ay * m.ir;
+    }
+    m.ux = MC == MODEL_CAVITY ? jx * m.ir : mad(jx, m.ir, ax);
+    m.uy = mad(jy, m.ir, ay);
+    const R hx = MC == MODEL_CAVITY ? R(-0.5) * m.ux : mad(R(-0.5), m.ux, ax), hy = mad(R(-0.5), m.uy, ay);
+    m.T_d = mad(m.ux, hx, mad(m.uy, hy, mad(-P.E0, rho_d, sg) * m.ir)) * P.inv_Cv;
     mac_qe<MC>(m);
     m.rhoE_d = mad(R(0.5), m.qe, sg);
-    R E_d = mad(-P.E0, rho_d, m.rhoE_d) * m.ir;
-    m.T_d = mad(R(-0.5), mad(m.ux, m.ux, m.uy * m.uy), E_d) * P.inv_Cv;
     m.T = P.T0 + m.T_d;
     m.p_d = eos_dev<MC>(P, rho_d, m.rho, m.T_d, m.T);
     mac_tail(P, m);
@@ -279,11 +287,11 @@ LBM_HD void macros(const Params<R>& P, R rho_d, R jx, R jy, R sg, Mac<R>& m) {
 template <typename R>
 LBM_HD void compress(const Mac<R>& m, MacC<R>& c) {
     c.rho_d = m.rho_d; c.ir = m.ir; c.ux = m.ux; c.uy = m.uy;
-    c.rhoE_d = m.rhoE_d; c.T_d = m.T_d; c.p_d = m.p_d;
+    c.T_d = m.T_d; c.p_d = m.p_d;
 }
 
 template <int MC = MODEL_ANY, typename R>
-LBM_HD void expand(const Params<R>& P, const MacC<R>& c, Mac<R>& m) {
+LBM_HD void expand(const Params<R>& P, const MacC<R>& c, R sg, Mac<R>& m) {
     m.rho_d = c.rho_d;
     m.rho = P.rho0 + c.rho_d;
     m.ir = c.ir;
@@ -291,7 +299,7 @@ LBM_HD void expand(const Params<R>& P, const MacC<R>& c, Mac<R>& m) {
     m.ux = c.ux;
     m.uy = c.uy;
     mac_qe<MC>(m);
-    m.rhoE_d = c.rhoE_d;
+    m.rhoE_d = mad(R(0.5), m.qe, sg);
     m.T_d = c.T_d;
     m.T = P.T0 + c.T_d;
     m.p_d = c.p_d;
@@ -755,12 +763,16 @@ LBM_HD void equilibrium(const Params<R>& P, const Mac<R>& mb, R* f, R* g) {
 // Sums over the 9 populations of a node: rho', j, sum g'.  Added in the order
 // of moments(), so that a kernel that calls both adds once.
 template <typename R>
+LBM_HD R sum9(const R* f) {
+    return f[0] + (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
+}
+template <typename R>
 LBM_HD void node_sums(const R* f, const R* g, R& rd, R& jx, R& jy, R& sg) {
     const R d1 = f[5] - f[7], d2 = f[6] - f[8];
-    rd = f[0] + (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
+    rd = sum9(f);
     jx = (f[1] - f[3]) + (d1 - d2);
     jy = (f[2] - f[4]) + (d1 + d2);
-    sg = g[0] + (((g[1] + g[3]) + (g[2] + g[4])) + ((g[5] + g[7]) + (g[6] + g[8])));
+    sg = sum9(g);
 }
 
 }  // namespace lbm
