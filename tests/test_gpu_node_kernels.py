@@ -29,6 +29,9 @@ def configs(precision):
     yield W.cavity(N=186, Ra=1e5, eps=0.4, eos=(W.EOS_CUBIC, (0.05, 0.2)), **p)   # cavity-model instance
     yield W.cavity(N=40, Ra=1e4, eps=0.1, order=2, tau0=0.8, **p)
     yield W.couette_variable_mu(nx=1, ny=32, **p)
+    yield W.periodic_box(64, 64, **p)                                             # most nodes of one cluster in FP32
+    yield W.cavity(N=65, Ra=1e4, eps=0.3, **p)                                    # one row and column beyond
+    yield W.poiseuille(nx=16, ny=128, **p)                                        # most nodes of one cluster in FP64
     yield W.poiseuille(nx=4, ny=128, **p)
     yield W.poiseuille(nx=200, ny=61, Th=1.01, **p)
     c = W.periodic_box(37, 29, **p)                                               # walls in x, periodic in y
@@ -54,7 +57,7 @@ def test_node_kernels_equal_strips(lbm, precision):
         for lat in (a, b, c):
             start(lat, cfg, 100 + k)
             lat.step(7)
-            lat.step(4)
+            lat.step(300 if 1 < cfg["nx"] < 40 else 4)   # 300: more than one cluster launch
             lat.sync()
         for x, y in zip(a.get_state(), b.get_state()):
             assert np.array_equal(x, y), (k, cfg["nx"], cfg["ny"])
