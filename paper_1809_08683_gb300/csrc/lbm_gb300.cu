@@ -2260,26 +2260,34 @@ __global__ void k_init_macros(const InstDesc* D, int b, const double* __restrict
     }
 }
 
-// plane q of buffer b <-> dense FP64 array [ny][nx] of full values (deviation + rest)
+// planes q0 .. q0 + gridDim.y - 1 of buffer b <-> dense FP64 arrays [ny][nx]
+// of full values (deviation + rest), one after another
+struct PlaneRests {
+    double rest[5];
+};
 template <typename R>
-__global__ void k_get_plane(const InstDesc* D, int b, int q, double rest, double* __restrict__ out) {
-    const long long nn = (long long)D->nx * D->ny;
-    const R* base = reinterpret_cast<const R*>(D->buf[b]) + q * D->plane;
+__global__ void k_get_planes(const InstDesc* D, int b, int q0, PlaneRests rests, double* __restrict__ out) {
+    const int nx = D->nx;
+    const long long nn = (long long)nx * D->ny;
+    const R* base = reinterpret_cast<const R*>(D->buf[b]) + (q0 + blockIdx.y) * D->plane;
+    const double rest = rests.rest[blockIdx.y];
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nn;
          t += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(t / D->nx), x = (int)(t % D->nx);
-        out[t] = (double)base[(long long)y * D->pitch + x] + rest;
+        const int y = (int)t / nx, x = (int)t - y * nx;
+        out[blockIdx.y * nn + t] = (double)base[(long long)y * D->pitch + x] + rest;
     }
 }
 
 template <typename R>
-__global__ void k_set_plane(const InstDesc* D, int b, int q, double rest, const double* __restrict__ in) {
-    const long long nn = (long long)D->nx * D->ny;
-    R* base = reinterpret_cast<R*>(D->buf[b]) + q * D->plane;
+__global__ void k_set_planes(const InstDesc* D, int b, int q0, PlaneRests rests, const double* __restrict__ in) {
+    const int nx = D->nx;
+    const long long nn = (long long)nx * D->ny;
+    R* base = reinterpret_cast<R*>(D->buf[b]) + (q0 + blockIdx.y) * D->plane;
+    const double rest = rests.rest[blockIdx.y];
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nn;
          t += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(t / D->nx), x = (int)(t % D->nx);
-        base[(long long)y * D->pitch + x] = (R)(in[t] - rest);
+        const int y = (int)t / nx, x = (int)t - y * nx;
+        base[(long long)y * D->pitch + x] = (R)(in[blockIdx.y * nn + t] - rest);
     }
 }
 
@@ -3961,36 +3969,55 @@ lbm_status lbm_macros(lbm_ctx* c, double* rho, double* ux, double* uy, double* T
     return c->sticky;
 }
 
+// The runs of planes that state transfers move at once: f and then g in runs
+// of at most five, as many as the staging area holds.  Each run is one copy
+// and one kernel, ordered by the stream alone; a copy and a synchronisation
+// per plane were 0.41 ms (set) and 0.32 ms (get) of a 193 x 150 FP64 lattice.
+extern "C++" {
+template <typename F>
+static lbm_status each_plane_run(const lbm_ctx* c, F&& run) {
+    for (int q0 : {0, 5, 9, 14}) {
+        const int n = (q0 == 0 || q0 == 9) ? 5 : 4;
+        PlaneRests r{};
+        for (int i = 0; i < n; ++i) r.rest[i] = q0 < 9 ? c->f_rest[q0 + i] : c->g_rest[q0 - 9 + i];
+        lbm_status st = run(q0, n, r);
+        if (st != LBM_OK) return st;
+    }
+    return LBM_OK;
+}
+}
+
 lbm_status lbm_get_state(lbm_ctx* c, double* f, double* g) {
     if (!c || !c->eos_set) return fail(LBM_EINVAL, "context not initialised");
     const long long nn = (long long)c->cfg.nx * c->cfg.ny;
-    for (int q = 0; q < 18; ++q) {
-        double* host = q < 9 ? (f ? f + q * nn : nullptr) : (g ? g + (q - 9) * nn : nullptr);
-        if (!host) continue;
-        const double rest = q < 9 ? c->f_rest[q] : c->g_rest[q - 9];
-        if (is_fp32(c)) k_get_plane<float><<<grid_for(nn), 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q, rest, c->d_stage);
-        else k_get_plane<double><<<grid_for(nn), 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q, rest, c->d_stage);
-        lbm_status st = check_launch();
-        if (st != LBM_OK) return st;
-        CUDA_TRY(cudaMemcpyAsync(host, c->d_stage, nn * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(cudaStreamSynchronize(c->stream));
-    }
+    lbm_status st = each_plane_run(c, [&](int q0, int n, const PlaneRests& r) {
+        double* host = q0 < 9 ? (f ? f + q0 * nn : nullptr) : (g ? g + (q0 - 9) * nn : nullptr);
+        if (!host) return LBM_OK;
+        const dim3 grid((unsigned)grid_for(nn), (unsigned)n);
+        if (is_fp32(c)) k_get_planes<float><<<grid, 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q0, r, c->d_stage);
+        else k_get_planes<double><<<grid, 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q0, r, c->d_stage);
+        lbm_status s = check_launch();
+        if (s != LBM_OK) return s;
+        CUDA_TRY(cudaMemcpyAsync(host, c->d_stage, n * nn * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        return LBM_OK;
+    });
+    if (st != LBM_OK) return st;
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
     return LBM_OK;
 }
 
 lbm_status lbm_set_state(lbm_ctx* c, const double* f, const double* g) {
     if (!c || !c->eos_set || !f || !g) return fail(LBM_EINVAL, "context not initialised or null state");
     const long long nn = (long long)c->cfg.nx * c->cfg.ny;
-    for (int q = 0; q < 18; ++q) {
-        const double* host = q < 9 ? f + q * nn : g + (q - 9) * nn;
-        const double rest = q < 9 ? c->f_rest[q] : c->g_rest[q - 9];
-        CUDA_TRY(cudaMemcpyAsync(c->d_stage, host, nn * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-        if (is_fp32(c)) k_set_plane<float><<<grid_for(nn), 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q, rest, c->d_stage);
-        else k_set_plane<double><<<grid_for(nn), 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q, rest, c->d_stage);
-        lbm_status st = check_launch();
-        if (st != LBM_OK) return st;
-        CUDA_TRY(cudaStreamSynchronize(c->stream));
-    }
+    lbm_status st = each_plane_run(c, [&](int q0, int n, const PlaneRests& r) {
+        const double* host = q0 < 9 ? f + q0 * nn : g + (q0 - 9) * nn;
+        CUDA_TRY(cudaMemcpyAsync(c->d_stage, host, n * nn * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+        const dim3 grid((unsigned)grid_for(nn), (unsigned)n);
+        if (is_fp32(c)) k_set_planes<float><<<grid, 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q0, r, c->d_stage);
+        else k_set_planes<double><<<grid, 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q0, r, c->d_stage);
+        return check_launch();
+    });
+    if (st != LBM_OK) return st;
     CUDA_TRY(cudaMemsetAsync(c->d_status, 0, 256, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     c->sticky = LBM_OK;
