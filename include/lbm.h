@@ -204,7 +204,7 @@ lbm_status lbm_peak_rates(void* cuda_stream, double* out3);
  * strips of 60 columns, two neighbouring nodes per lane in packed FP32,
  * bx = 60, 120 or 240.  pair = 6: node kernels, one launch that collides
  * and pushes every node and one that rebuilds the wall nodes and writes every
- * node's macros for the next step; bx = 128 nodes per CTA, by has no effect,
+ * node's macros for the next step; bx = 128 by name, by has no effect,
  * any precision.  pair = 0, 4 and 6 shapes of any width give identical
  * results; pairs 1-3 and 5 agree with them to FP32 rounding (pairs 1, 2 and
  * 5 draw one random number per two nodes).  (bx, by, pair) = (0, 0, 0)

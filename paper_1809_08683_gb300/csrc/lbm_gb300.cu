@@ -1817,7 +1817,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? LBM_BOUNDARY_MINB : 2) k
 // ------------------------------------------------------------------------
 
 // A step of a lattice whose DFs stay in L2, or whose arithmetic is FP64, as
-// two launches over all its nodes in row-major order, 128 per CTA:
+// two launches over all its nodes in row-major order:
 //   k_collide_node   collides and pushes every node; rho' and p' of its
 //                    neighbours come from the lattice's field array;
 //   k_prep           rebuilds the wall nodes of the buffer pushed into (what
@@ -1849,10 +1849,18 @@ struct Field {
         return RhoP<R>{v.x, v.y};
     }
 };
-constexpr int kNodeThreads = 128;
+// Threads per CTA: 64, which spreads a small lattice over twice the SMs of 128
+// (us per step of a cavity: FP64 150^2 49.9 -> 41.5, 256^2 72.9 -> 69.7; FP32
+// 256^2 9.9 -> 9.4, 512^2 16.4 -> 15.7), but 128 for the one-node FP32 collision,
+// whose CTAs are short (512^2 FP32 channel 17.1 us, with 64 18.0).
+template <typename R>
+struct NodeThreads {
+    static constexpr int collide = sizeof(R) == 4 ? 128 : 64, prep = 64;
+};
+constexpr int kPairThreads = 64;
 
-__host__ __device__ inline int node_ctas(long long n, int per_cta = kNodeThreads) { return (int)((n + per_cta - 1) / per_cta); }
-__host__ __device__ inline int wall_per_cta(int pairs) { return pairs ? kNodeThreads / 2 : kNodeThreads; }
+__host__ __device__ inline int node_ctas(long long n, int per_cta) { return (int)((n + per_cta - 1) / per_cta); }
+__host__ __device__ inline int wall_per_cta(int threads, int pairs) { return pairs ? threads / 2 : threads; }
 __device__ __forceinline__ NWork node_item(int block, long long n0, long long end, int per_cta, int kind) {
     const long long first = n0 + (long long)block * per_cta;
     return NWork{0, (int)first, (int)min((long long)per_cta, end - first), kind, 0, 0};
@@ -1870,7 +1878,7 @@ __device__ __forceinline__ NWork collide_work(const NWork* __restrict__ work, In
 __device__ __forceinline__ NWork prep_work(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta) {
     if (work) return work[blockIdx.x];
     const InstDesc* D = descs[0];
-    const int per_wall = wall_per_cta(D->wall_pairs), kind = D->wall_pairs ? kWallPairs : kWallNodes;
+    const int per_wall = wall_per_cta((int)blockDim.x, D->wall_pairs), kind = D->wall_pairs ? kWallPairs : kWallNodes;
     const int nwall = wall_count(D->nx, D->ny, D->px, D->py), wall_ctas = node_ctas(nwall, per_wall), edge = D->py ? 0 : 1;
     if ((int)blockIdx.x < wall_ctas) return node_item(blockIdx.x, 0, nwall, per_wall, kind);
     return node_item(blockIdx.x - wall_ctas, (long long)D->nx * edge, (long long)D->nx * (D->ny - edge), per_cta, kInnerNodes);
@@ -1899,7 +1907,7 @@ __device__ __forceinline__ void prep_inner(const NWork& w, const InstDesc* D, co
     if ((!D->px && (x == 0 || x == nx - 1)) || (!D->py && (y == 0 || y == ny - 1))) return;
     R v[18];
     load18<R, CG>(buf, D->plane, (long long)y * D->pitch + x, v);
-    put_macros(D, P, v, x, y, !CG && i + kNodeThreads >= w.cnt);
+    put_macros(D, P, v, x, y, !CG && i + NodeThreads<R>::prep >= w.cnt);
 }
 template <typename R, bool CG = false>
 __device__ __forceinline__ void prep_wall(const NWork& w, const InstDesc* D, const Params<R>& P, R* buf, int wall_mode, int i) {
@@ -1935,16 +1943,16 @@ __device__ __forceinline__ void prep_wall_pairs(const InstDesc* D, const Params<
     put_macros(D, P, v, n.x, n.y, !CG);
 }
 
-// Six CTAs per SM in FP32, at the price of a few spills on the wall path: 64
-// small lattices take 26.5 us per step against 27.6 us with four, 768^2 27.4
+// 24 warps per SM in FP32, at the price of a few spills on the wall path: 64
+// small lattices take 26.5 us per step against 27.6 us with 16, 768^2 27.4
 // against 29.0; FP64 keeps its registers, whose spills would lengthen the
-// wall nodes' serial work (256^2: 74 us per step with two, 76 with three).
+// wall nodes' serial work (256^2: 74 us per step with 8 warps, 76 with 12).
 // The two kinds of item share no code path: one common tail cost the inner
 // nodes their batched loads (64 small lattices 29.1 us).  PAIRS: some wall of
 // some lattice extrapolates to second order; the instance without that path
 // is 1.3% faster on a 512^2 FP64 cavity and 1.5% on a 768^2 FP32 one.
 template <typename R, bool PAIRS>
-__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 6 : 2)
+__global__ void __launch_bounds__(NodeThreads<R>::prep, sizeof(R) == 4 ? 12 : 4)
     k_prep(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta, int step_par, int wall_mode,
            long long* counter) {
     __shared__ Params<R> P;
@@ -1961,7 +1969,7 @@ __global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 6 : 2)
     } else if (w.kind == kWallNodes) {
         if ((int)threadIdx.x < w.cnt) prep_wall(w, D, P, buf, wall_mode, threadIdx.x);
     } else {
-        for (int i = threadIdx.x; i < w.cnt; i += kNodeThreads) prep_inner(w, D, P, buf, i);
+        for (int i = threadIdx.x; i < w.cnt; i += NodeThreads<R>::prep) prep_inner(w, D, P, buf, i);
     }
 }
 
@@ -2031,12 +2039,12 @@ __device__ __forceinline__ void collide_node(const NWork& w, const InstDesc* D, 
     if (!(lbm::finite(m.rho_d) && lbm::finite(m.T_d))) atomicOr(D->status, 1u);
     AddDither add(mix32(step_hash ^ ((uint32_t)y * 0x85ebca77u + (uint32_t)x * 0xc2b2ae3du)), (float)P.dither);
     lbm::collide<MC>(P, m, v, v + 9, grx, gry, gpx, gpy, add);
-    if (!CG && i + kNodeThreads >= w.cnt) let_next_start();
+    if (!CG && i + NodeThreads<R>::collide >= w.cnt) let_next_start();
     push_node(dst, v, x, y, nx, ny, pitch, plane, px, py);
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 5 : 2)
+__global__ void __launch_bounds__(NodeThreads<R>::collide, sizeof(R) == 4 ? 5 : 4)
     k_collide_node(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta, int step_par,
                    const long long* counter) {
     __shared__ Params<R> P;
@@ -2046,7 +2054,7 @@ __global__ void __launch_bounds__(kNodeThreads, sizeof(R) == 4 ? 5 : 2)
     __syncthreads();
     wait_for_previous();
     const uint32_t step_hash = mix32((uint32_t)(w.step0 + *counter) * 0x9e3779b1u + 0x632be5abu);
-    for (int i = threadIdx.x; i < w.cnt; i += kNodeThreads) {
+    for (int i = threadIdx.x; i < w.cnt; i += NodeThreads<R>::collide) {
         if (D->mc == lbm::MODEL_CAVITY) collide_node<R, lbm::MODEL_CAVITY>(w, D, P, step_par, step_hash, i);
         else collide_node<R, lbm::MODEL_ANY>(w, D, P, step_par, step_hash, i);
     }
@@ -2194,11 +2202,11 @@ __device__ __forceinline__ void collide_node2(const NWork& w, const InstDesc* D,
         atomicOr(D->status, 1u);
     AddDither2 add(mix32(step_hash ^ ((uint32_t)y * 0x85ebca77u + (uint32_t)xa * 0xc2b2ae3du)), dscale);
     lbm::collide<MC>(P, mf, v, v + 9, grx, gry, gpx, gpy, add);
-    if (i + kNodeThreads >= w.cnt) let_next_start();
+    if (i + kPairThreads >= w.cnt) let_next_start();
     push_pair(dst, v, xa, act_b, y, nx, ny, pitch, plane, px, py);
 }
 
-__global__ void __launch_bounds__(kNodeThreads, 3)
+__global__ void __launch_bounds__(kPairThreads, 6)
     k_collide_node2(const NWork* __restrict__ work, InstDesc* const* __restrict__ descs, int per_cta, int step_par,
                     const long long* counter) {
     __shared__ Params<f2> P;
@@ -2208,12 +2216,12 @@ __global__ void __launch_bounds__(kNodeThreads, 3)
     constexpr int nf = offsetof(Params<float>, eos) / sizeof(float);
     static_assert(offsetof(Params<f2>, eos) == nf * sizeof(f2), "Params is numbers, then integers");
     const float* pf = reinterpret_cast<const float*>(&D->pf);
-    for (int i = threadIdx.x; i < nf; i += kNodeThreads) reinterpret_cast<float2*>(&P)[i] = make_float2(pf[i], pf[i]);
+    for (int i = threadIdx.x; i < nf; i += kPairThreads) reinterpret_cast<float2*>(&P)[i] = make_float2(pf[i], pf[i]);
     if (threadIdx.x < 4) reinterpret_cast<int*>(&P.eos)[threadIdx.x] = reinterpret_cast<const int*>(&D->pf.eos)[threadIdx.x];
     __syncthreads();
     wait_for_previous();
     const uint32_t step_hash = mix32((uint32_t)(w.step0 + *counter) * 0x9e3779b1u + 0x632be5abu);
-    for (int i = threadIdx.x; i < w.cnt; i += kNodeThreads) {
+    for (int i = threadIdx.x; i < w.cnt; i += kPairThreads) {
         if (D->mc == lbm::MODEL_CAVITY) collide_node2<lbm::MODEL_CAVITY>(w, D, P, D->pf.dither, step_par, step_hash, i);
         else collide_node2<lbm::MODEL_ANY>(w, D, P, D->pf.dither, step_par, step_hash, i);
     }
@@ -2967,16 +2975,18 @@ void ensure_tick(std::vector<BWork>& v, int inst, int par) {
     }
 }
 
-// Nodes (or pairs) per CTA of a node kernel: 128, and up to `most` times as
-// many where the launch would otherwise be more than one fill of the GPU, so
+// Nodes (or pairs) per CTA of a node kernel: one per thread, and up to `most`
+// times as many where the launch would otherwise be more than one fill of the GPU, so
 // that a CTA's set-up (work item, descriptor, parameters) serves more nodes.
 // Two in FP32 (64 small lattices: 27.3 us per step against 29.2 us with one
 // and 29.0 us with four) but one for pairs, and four for k_prep in FP64, where
 // one tile is 51 instructions (298 us against 305 us), against one for the
 // collision, whose 320 want an even load (298 us against 316 us with two).
-int per_cta_for(long long nodes, int ctas_per_sm, int most) {
-    const long long tiles = nodes / ((long long)kNodeThreads * 152 * ctas_per_sm);
-    return kNodeThreads * (int)std::max<long long>(1, std::min<long long>(most, tiles));
+// Beyond 64 fills the load is even anyway, and more nodes per CTA keep a
+// batch's table short (64 FP64 lattices of 2048^2: 60,000 items, not 4 million).
+int per_cta_for(long long nodes, int threads, int ctas_per_sm, int most) {
+    const long long fills = nodes / ((long long)threads * 152 * ctas_per_sm);
+    return threads * (int)std::max({1LL, std::min<long long>(most, fills), fills / 64});
 }
 
 // Work items of the node kernels for one lattice: every node for
@@ -2987,6 +2997,7 @@ void add_node_work(const lbm_config& c, int inst, int par, bool pairs, long long
     for (long long n0 = 0; n0 < nn; n0 += per_cta)
         v.push_back(NWork{inst, (int)n0, (int)std::min<long long>(per_cta, nn - n0), kInnerNodes, par, step0});
 }
+int prep_threads(bool fp32) { return fp32 ? NodeThreads<float>::prep : NodeThreads<double>::prep; }
 int wall_pairs(const lbm_config& c) {
     for (const lbm_wall_bc& w : c.wall)
         if (!w.periodic && w.extrap_order == 2) return 1;
@@ -2994,7 +3005,7 @@ int wall_pairs(const lbm_config& c) {
 }
 void add_prep_wall(const lbm_config& c, int inst, int par, std::vector<NWork>& v) {
     const int n = wall_count(c.nx, c.ny, c.wall[LBM_WALL_W].periodic != 0, c.wall[LBM_WALL_S].periodic != 0);
-    const int pairs = wall_pairs(c), per = wall_per_cta(pairs);
+    const int pairs = wall_pairs(c), per = wall_per_cta(prep_threads(c.precision == LBM_FP32_DEV), pairs);
     for (int n0 = 0; n0 < n; n0 += per)
         v.push_back(NWork{inst, n0, std::min(per, n - n0), pairs ? kWallPairs : kWallNodes, par, 0});
 }
@@ -3018,10 +3029,16 @@ bool node_kernels(const lbm_ctx* c, long long nodes) {
 // Which of them: 0 FP64, 1 FP32, 2 FP32 in pairs (lattices whose strips are paired).
 enum { kNode64 = 0, kNode32 = 1, kNodePair = 2, kNodeKinds = 3 };
 int node_kind(const lbm_ctx* c) { return c->cfg.precision == LBM_FP64 ? kNode64 : c->pair == 1 ? kNodePair : kNode32; }
-int collide_per_cta(int kind, long long nodes) {
-    return kind == kNode32 ? per_cta_for(nodes, 5, 2) : kNodeThreads;
+int node_threads(int kind) {
+    return kind == kNode32 ? NodeThreads<float>::collide : kind == kNode64 ? NodeThreads<double>::collide : kPairThreads;
 }
-int prep_per_cta(bool fp32, long long nodes) { return fp32 ? per_cta_for(nodes, 5, 2) : per_cta_for(nodes, 2, 4); }
+int collide_per_cta(int kind, long long nodes) {
+    if (kind == kNode32) return per_cta_for(nodes, node_threads(kind), 5, 2);
+    return per_cta_for(kind == kNodePair ? nodes / 2 : nodes, node_threads(kind), 6, 1);
+}
+int prep_per_cta(bool fp32, long long nodes) {
+    return fp32 ? per_cta_for(nodes, prep_threads(true), 640 / prep_threads(true), 2) : per_cta_for(nodes, prep_threads(false), 4, 4);
+}
 
 // Default launch shape.  Lattices up to 160 columns wide take warp strips
 // of 30 columns (pair 4, same bits as pair 0): they waste fewer lanes there
@@ -3136,15 +3153,25 @@ int cluster_ctas_for(long long nn) {
     if (nn > ClusterTraits<R>::max_nodes) return 0;
     int n = 1;
     while (n < ClusterTraits<R>::max_ctas && (long long)n * 32 < nn) n *= 2;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    cluster_config(cfg, at, n, cluster_threads(nn, n), nullptr);
-    int fit = 0;
-    if (cudaOccupancyMaxActiveClusters(&fit, k_steps_cluster<R>, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
+    // whether the device holds such a cluster, asked once per device and shape
+    // (the question takes about a quarter of a millisecond)
+    static std::mutex mu;
+    static signed char cache[64][ClusterTraits<R>::max_ctas + 1][ClusterTraits<R>::threads / 32 + 1] = {};
+    const int threads = cluster_threads(nn, n);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    signed char& known = cache[dev][n][threads / 32];
+    if (!known) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        cluster_config(cfg, at, n, threads, nullptr);
+        int fit = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, k_steps_cluster<R>, &cfg);
+        if (e != cudaSuccess) cudaGetLastError();
+        known = e == cudaSuccess && fit > 0 ? 1 : -1;
     }
-    return fit > 0 ? n : 0;
+    return known > 0 ? n : 0;
 }
 constexpr int kClusterSteps = 256;  // most steps of one launch
 template <typename R>
@@ -3165,7 +3192,7 @@ lbm_status upload_work(lbm_ctx* c) {
         c->node_per_cta = collide_per_cta(node_kind(c), (long long)nx * ny);
         c->prep_per_cta = prep_per_cta(is_fp32(c), (long long)nx * ny);
         c->n_node = node_ctas((long long)(node_kind(c) == kNodePair ? (nx + 1) / 2 : nx) * ny, c->node_per_cta);
-        c->n_prep = node_ctas(wall_count(nx, ny, c->h.px, c->h.py), wall_per_cta(c->h.wall_pairs)) + node_ctas((long long)nx * (ny - 2 * edge), c->prep_per_cta);
+        c->n_prep = node_ctas(wall_count(nx, ny, c->h.px, c->h.py), wall_per_cta(prep_threads(is_fp32(c)), c->h.wall_pairs)) + node_ctas((long long)nx * (ny - 2 * edge), c->prep_per_cta);
         c->cluster_ctas = is_fp32(c) ? cluster_ctas_for<float>((long long)nx * ny) : cluster_ctas_for<double>((long long)nx * ny);
         return LBM_OK;
     }
@@ -3377,7 +3404,7 @@ void launch_pair_bx(const Work* work, int n, InstDesc* const* descs, int par, co
 }
 
 static const int kVariantWidth[kVariants] = {32, 64, 128, 64, 128, 256, 64, 128, 256, 32, 64, 128, 30, 60, 120,
-                                            60, 120, 240, kNodeThreads};
+                                            60, 120, 240, 128};
 static const int kVariantPair[kVariants] = {0, 0, 0, 1, 1, 1, 2, 2, 2, 3, 3, 3, 4, 4, 4, 5, 5, 5, 6};
 
 int variant_index(int bx, int pair) {
@@ -3450,14 +3477,14 @@ void launch_boundary(const BWork* work, int n, InstDesc* const* descs, int par, 
 
 void launch_node(int kind, const NWork* work, int n, int per_cta, InstDesc* const* descs, int par, const long long* counter, cudaStream_t s) {
     if (n <= 0) return;
-    if (kind == kNodePair) launch_step(k_collide_node2, n, kNodeThreads, 0, s, work, descs, per_cta, par, counter);
-    else if (kind == kNode32) launch_step(k_collide_node<float>, n, kNodeThreads, 0, s, work, descs, per_cta, par, counter);
-    else launch_step(k_collide_node<double>, n, kNodeThreads, 0, s, work, descs, per_cta, par, counter);
+    if (kind == kNodePair) launch_step(k_collide_node2, n, node_threads(kind), 0, s, work, descs, per_cta, par, counter);
+    else if (kind == kNode32) launch_step(k_collide_node<float>, n, node_threads(kind), 0, s, work, descs, per_cta, par, counter);
+    else launch_step(k_collide_node<double>, n, node_threads(kind), 0, s, work, descs, per_cta, par, counter);
 }
 void launch_prep(bool fp32, bool pairs, const NWork* work, int n, int per_cta, InstDesc* const* descs, int par, int wall_mode, long long* counter,
                  cudaStream_t s) {
     if (n <= 0) return;
-    auto go = [&](auto kernel) { launch_step(kernel, n, kNodeThreads, 0, s, work, descs, per_cta, par, wall_mode, counter); };
+    auto go = [&](auto kernel) { launch_step(kernel, n, prep_threads(fp32), 0, s, work, descs, per_cta, par, wall_mode, counter); };
     if (fp32) pairs ? go(k_prep<float, true>) : go(k_prep<float, false>);
     else pairs ? go(k_prep<double, true>) : go(k_prep<double, false>);
 }

@@ -493,16 +493,6 @@ LBM_HD void heating(R ux, R uy, R v1, R v7, R v8, R& Y3, R& Y5) {
     Y5 = mad(uy, b, ux * c);
 }
 
-// Plain update: new = old + delta, rounded to nearest, for the pair
-// (f_i, g_i) of one link.
-struct AddNearest {
-    template <typename R>
-    LBM_HD void operator()(R& f, R df, R& g, R dg) const {
-        f = f + df;
-        g = g + dg;
-    }
-};
-
 // Leaves f and g as they are between the moments and the final update.
 struct KeepDFs {
     template <typename R>
@@ -632,11 +622,6 @@ LBM_HD void collide(const Params<R>& P, const Mac<R>& mc, R* f, R* g, R rx, R ry
     reload(f, g);
 #pragma unroll
     for (int i = 0; i < 9; ++i) add(f[i], df[i], g[i], dg[i]);
-}
-
-template <typename R>
-LBM_HD void collide(const Params<R>& P, const Mac<R>& mc, R* f, R* g, R rx, R ry, R px, R py) {
-    collide(P, mc, f, g, rx, ry, px, py, AddNearest());
 }
 
 // Redefined non-equilibrium moments of Eq. (neq.redefinition) at a fluid

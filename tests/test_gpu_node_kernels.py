@@ -92,3 +92,17 @@ def test_batch_of_node_and_strip_members_equals_alone(lbm, graph_steps):
         assert all(np.array_equal(p, q) for p, q in zip(x.get_state(), y.get_state()))
         assert x.steps == y.steps == 12
     batch.close()
+
+
+@pytest.mark.parametrize("cfg", [W.poiseuille(nx=499, ny=421, precision=1), W.cavity(N=520, Ra=1e6, eps=0.5, precision=0)],
+                         ids=["fp32", "fp64-prep"])
+def test_several_tiles_per_cta(lbm, cfg):
+    a, b = lbm.Lattice(cfg), lbm.Lattice(cfg)
+    b.set_tile(64, 8, 0)
+    for lat in (a, b):
+        lat.init_macros(*W.random_macros(cfg["nx"], cfg["ny"], 3))
+        lat.step(3)
+    for x, y in zip(a.get_state(), b.get_state()):
+        assert np.array_equal(x, y)
+    a.close()
+    b.close()
