@@ -22,6 +22,15 @@
 // (k_collide_pair: two nodes per thread in packed FP32) and paired warp
 // strips (k_collide_warp2); default_shape picks one per lattice and
 // lbm_set_tile selects any other.
+//
+// FP64 lattices, and FP32 ones of few nodes, step with the same bits through
+// two other kernels (node_kernels says when):
+//   k_prep           : rebuilds the wall nodes and writes every node's
+//                      macros to a field array;
+//   k_collide_node   : collides and pushes one node per thread in row-major
+//                      order (k_collide_node2: two, for paired lattices).
+// k_steps_cluster runs both for many steps of a lattice that fits one
+// thread-block cluster.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -418,8 +427,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
 // __restrict__: the compiler may move such a read-only load over the wait,
 // and the data is not read-only for as long as the kernel is resident.
 // The node kernels and the wall pass let the next one start just before
-// their stores: a lone 256^2 FP32 cavity takes 10.3 us per step against
-// 16.4 us without (64^2: 8.2 against 14.4; 512^2 FP64: 202 against 208).
+// their stores: a lone 256^2 FP32 cavity took 10.3 us per step against
+// 16.4 us without (512^2 FP64: 202 against 208; 9.3 and 193 now).
 // At their beginning would be worse for lattices that fill the GPU: the next
 // kernel's CTAs then settle wherever slots are free and load the SMs
 // unevenly (193 x 150 FP64: 74 us against 58 us per step).  The strips never
@@ -2855,14 +2864,19 @@ constexpr int kModels = 2;  // model classes: lbm::MODEL_ANY, lbm::MODEL_CAVITY
 // cavity model: they are latency-bound, and batches of them (the serving
 // mix) then stay one launch per shape.
 constexpr long long kModelMinNodes = 32768;
-// Most FP32 nodes that default shapes step through the node kernels.  Beyond
-// about this many their second read of the DFs, 72 B per node, no longer
-// comes from L2.  us per step of a lone cavity, node kernels and strips:
-// 512^2 17 and 25, 768^2 33 and 37, 1024^2 65 and 56; of a periodic box: 19
-// and 22, 39 and 40, 77 and 56.
+// Most FP32 nodes that default shapes step through the node kernels, counted
+// over the lattices stepped together whose strips would be block strips (the
+// paired ones among them).  Beyond about this many the second read of the DFs,
+// 72 B per node, no longer comes from L2.  us per step of a lone cavity, node
+// kernels and strips: 512^2 16 and 25, 768^2 28 and 37, 1024^2 65 and 49; of a
+// periodic box: 17 and 22, 31 and 40, 77 and 56.  Lattices of up to 160
+// columns, whose warp strips leave more idle, gain up to more nodes: batches
+// of 64 to 128 a side take 61 and 45 us (strips, node kernels) at 0.6M nodes,
+// 132 and 115 at 1.5M, 245 and 249 at 3.1M.
 #ifndef LBM_NODE_MAX_FP32
 #define LBM_NODE_MAX_FP32 600000
 #endif
+constexpr long long kNodeMaxNarrow = 2500000;
 constexpr long long kNodeMaxFp32 = LBM_NODE_MAX_FP32;
 
 // The launches of one time step over a set of members: launch groups
@@ -2927,8 +2941,8 @@ std::vector<Work> make_work(const lbm_config& c, int inst, int bx, int by, int p
 // The last `resident` work items (one fill of the GPU) are cut into up to
 // four runs of at least 6 rows each (shorter runs re-stage too many halo
 // rows), placed last; that shortens the idle end to about a quarter of a
-// run.  Measured on the 96-cavity batch (runs of 32 rows): fused launch
-// 1.138 -> 1.123 ms; 16 cavities of 1024^2: 0.503 -> 0.488 ms.  Which CTA
+// run.  Measured on the 96-cavity batch (runs of 32 rows) when it went in:
+// fused launch 1.138 -> 1.123 ms; 16 cavities of 1024^2: 0.503 -> 0.488 ms.  Which CTA
 // updates a node does not change its arithmetic, so the results are the
 // same bits.
 void split_tail(std::vector<Work>& v, long long resident) {
@@ -3020,11 +3034,17 @@ bool is_fp32(const lbm_ctx* c) { return c->cfg.precision == LBM_FP32_DEV; }
 
 // Whether a lattice steps through the node kernels: always when lbm_set_tile
 // chose them; with a default shape, FP64 lattices always, and FP32 lattices
-// while the nodes stepped together (`nodes`: one lattice, or a batch's FP32
-// members) are few enough.  See kNodeMaxFp32.
-bool node_kernels(const lbm_ctx* c, long long nodes) {
+// while the nodes of their class stepped together (`nodes`: one lattice, or a
+// batch's FP32 members with a default shape) are few enough.  See
+// kNodeMaxFp32.
+struct ClassNodes {
+    long long narrow = 0, wide = 0;  // default shape: warp strips, others
+    void add(const lbm_ctx* c) { (c->pair == 4 ? narrow : wide) += (long long)c->cfg.nx * c->cfg.ny; }
+};
+bool node_kernels(const lbm_ctx* c, const ClassNodes& nodes) {
     if (c->tile_set) return c->pair == 6;
-    return c->cfg.precision == LBM_FP64 || nodes <= kNodeMaxFp32;
+    if (c->cfg.precision == LBM_FP64) return true;
+    return c->pair == 4 ? nodes.narrow <= kNodeMaxNarrow : nodes.wide <= kNodeMaxFp32;
 }
 // Which of them: 0 FP64, 1 FP32, 2 FP32 in pairs (lattices whose strips are paired).
 enum { kNode64 = 0, kNode32 = 1, kNodePair = 2, kNodeKinds = 3 };
@@ -3044,10 +3064,9 @@ int prep_per_cta(bool fp32, long long nodes) {
 // of 30 columns (pair 4, same bits as pair 0): they waste fewer lanes there
 // and give small lattices more CTAs.  Wider FP32 lattices of the heated-
 // cavity model class take paired block strips of 128 columns (pair 1): two
-// nodes per thread in packed FP32 halve the arithmetic's issue slots (4096^2:
-// 0.49 ms against 0.55 ms for block strips; 96-cavity batch: 1.30 ms against
-// 1.39 ms per step).  All others take block strips of 128 columns (pair 0),
-// which also suit FP64, bound by the FP64 pipe.  The model class is known
+// nodes per thread in packed FP32 halve the arithmetic's issue slots (96-
+// cavity batch: 1.112 ms per step against 1.285 ms for block strips).  All
+// others take block strips of 128 columns (pair 0), in FP64 too.  The model class is known
 // once the EOS is set, so lbm_set_eos applies the shape.
 void default_shape(const lbm_config& c, int mc, int& bx, int& pair) {
     if (c.nx <= 160) { bx = 30; pair = 4; }
@@ -3059,7 +3078,7 @@ void default_shape(const lbm_config& c, int mc, int& bx, int& pair) {
 // 2048^2 (FP64) lattice and on the 96-cavity batch (longer runs lose DRAM
 // and L2 locality between CTAs resident at the same time, shorter ones
 // re-stage more halo rows).  Paired block strips: 32 rows on the 96-cavity
-// batch (1.285 ms per step against 1.302 ms with 24).
+// batch (1.113 ms per step against 1.123 ms with 24 and 1.118 ms with 48).
 int batch_rows(const lbm_config& c, int pair) {
     const bool f32 = c.precision == LBM_FP32_DEV;
     const int by = pair == 0 ? (f32 ? 24 : 8) : pair == 1 ? 32 : (pair == 5 ? 16 : 24);
@@ -3186,7 +3205,9 @@ void launch_cluster(InstDesc* const* descs, long long nn, int ctas, long nsteps,
 lbm_status upload_work(lbm_ctx* c) {
     if (c->d_work) { cudaFree(c->d_work); c->d_work = nullptr; }
     c->n_node = c->n_prep = c->cluster_ctas = 0;
-    if (node_kernels(c, (long long)c->cfg.nx * c->cfg.ny)) {
+    ClassNodes own;
+    own.add(c);
+    if (node_kernels(c, own)) {
         // no table: the kernels find a lone lattice's work by themselves
         const int nx = c->cfg.nx, ny = c->cfg.ny, edge = c->h.py ? 0 : 1;
         c->node_per_cta = collide_per_cta(node_kind(c), (long long)nx * ny);
@@ -4335,9 +4356,9 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int n, int graph_steps, lbm_ba
     lbm_batch* b = new lbm_batch();
     b->stream = ctxs[0]->stream;
     std::vector<InstDesc*> descs;
-    long long nodes32 = 0;  // FP32 members with a default shape
+    ClassNodes nodes32;  // FP32 members with a default shape
     for (int i = 0; i < n; ++i)
-        if (ctxs[i] && !ctxs[i]->tile_set && is_fp32(ctxs[i])) nodes32 += (long long)ctxs[i]->cfg.nx * ctxs[i]->cfg.ny;
+        if (ctxs[i] && !ctxs[i]->tile_set && is_fp32(ctxs[i])) nodes32.add(ctxs[i]);
     std::vector<char> node(n, 0);
     for (int i = 0; i < n; ++i) node[i] = ctxs[i] && node_kernels(ctxs[i], nodes32);
     // rows per run of the members whose shape was not set: the batch length,

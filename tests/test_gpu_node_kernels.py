@@ -106,3 +106,26 @@ def test_several_tiles_per_cta(lbm, cfg):
         assert np.array_equal(x, y)
     a.close()
     b.close()
+
+
+def test_narrow_members_beside_many_wide_nodes(lbm):
+    """More than 600,000 nodes of up to 160 columns beside as many wider ones:
+    node kernels and strips in one batch, against each in its strips alone."""
+    import torch
+    st = torch.cuda.Stream()
+    cfgs = [W.periodic_box(160, 2000, precision=1), W.poiseuille(nx=100, ny=3001, precision=1),
+            W.periodic_box(161, 3800, precision=1)]
+    alone = [lbm.Lattice(c, stream=st) for c in cfgs]
+    mixed = [lbm.Lattice(c, stream=st) for c in cfgs]
+    for k, (a, b) in enumerate(zip(alone, mixed)):
+        a.set_tile(*((30, 8, 4) if k < 2 else (128, 8, 0)))
+        for lat in (a, b):
+            lat.init_macros(*W.random_macros(cfgs[k]["nx"], cfgs[k]["ny"], 60 + k))
+    batch = lbm.Batch(mixed, graph_steps=2)
+    batch.step(4)
+    for a, b in zip(alone, mixed):
+        a.step(4)
+        assert all(np.array_equal(p, q) for p, q in zip(a.get_state(), b.get_state()))
+    batch.close()
+    for lat in alone + mixed:
+        lat.close()
