@@ -1025,7 +1025,7 @@ struct PairSmem {
 __device__ void broadcast_params(const Params<float>& a, Params<f2>& b) {
 #define BP(f) b.f = f2(a.f)
     BP(rho0); BP(T0); BP(E0); BP(Cv); BP(inv_Cv); BP(Rg); BP(eos_a); BP(eos_b); BP(p0); BP(rho0E0_p0);
-    BP(rho0Cp0); BP(mu0); BP(mu0S); BP(inv_T0); BP(visc_S); BP(lam_fac); BP(nu_e); BP(mu_j); BP(beta2);
+    BP(mu0); BP(mu0S); BP(inv_T0); BP(visc_S); BP(lam_fac); BP(nu_e); BP(mu_j); BP(x2r); BP(x2p); BP(n1T); BP(n2T);
     BP(kk); BP(hh); BP(bb); BP(bbm2); BP(omk); BP(k2h); BP(gamma1); BP(gamma2); BP(k11); BP(k17); BP(k18);
     BP(k71); BP(k77); BP(k81); BP(k88); BP(Fx); BP(Fy); BP(Fxh); BP(Fyh); BP(cs_b0); BP(dither);
 #undef BP
@@ -2799,7 +2799,7 @@ template <typename A, typename B>
 void convert_params(const Params<A>& a, Params<B>& b) {
 #define CP(f) b.f = (B)a.f
     CP(rho0); CP(T0); CP(E0); CP(Cv); CP(inv_Cv); CP(Rg); CP(eos_a); CP(eos_b); CP(p0); CP(rho0E0_p0);
-    CP(rho0Cp0); CP(mu0); CP(mu0S); CP(inv_T0); CP(visc_S); CP(lam_fac); CP(nu_e); CP(mu_j); CP(beta2);
+    CP(mu0); CP(mu0S); CP(inv_T0); CP(visc_S); CP(lam_fac); CP(nu_e); CP(mu_j); CP(x2r); CP(x2p); CP(n1T); CP(n2T);
     CP(kk); CP(hh); CP(bb); CP(bbm2); CP(omk); CP(k2h); CP(gamma1); CP(gamma2); CP(k11); CP(k17); CP(k18);
     CP(k71); CP(k77); CP(k81); CP(k88); CP(Fx); CP(Fy); CP(Fxh); CP(Fyh); CP(cs_b0); CP(dither);
 #undef CP
@@ -3724,7 +3724,6 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
     P.eos_b = b;
     P.p0 = p0;
     P.rho0E0_p0 = r0 * P.E0 + p0;
-    P.rho0Cp0 = r0 * Cp;
     P.mu0 = r0 * (k.tau0 - 0.5) * cs2;
     P.mu0S = P.mu0 * (1.0 + k.visc_p[0]);
     P.inv_T0 = 1.0 / T0;
@@ -3732,11 +3731,15 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
     P.lam_fac = Cp / k.Pr;
     const double coef = 2.0 / 3.0 + k.gamma1 / 2.0 + k.gamma2 / 3.0;
     if (!(coef > 0)) return fail(LBM_EINVAL, "gamma1, gamma2 give a non-positive conductivity factor");
-    P.mu_j = 2.0 * P.lam_fac / (coef * r0 * Cp);
+    P.mu_j = 4.0 * P.lam_fac / (coef * r0 * Cp);
     const double e_fac = 3.0 * k.bulk_ratio / w;  // (1/s_e - 1/2) / nu
     P.nu_e = 2.0 * e_fac;
     // alpha1 = -1, beta1 = 1, so that alpha2 = -(2 alpha1 + w + 1) / (1 - w) = 1
-    P.beta2 = -2.0 / (1.0 - w);
+    const double beta2 = -2.0 / (1.0 - w);
+    P.x2r = beta2 - 1.0;
+    P.x2p = -3.0 * beta2;
+    P.n1T = -(4.0 + k.gamma1) * r0 * Cp;
+    P.n2T = (4.0 - k.gamma2) * r0 * Cp;
     P.kk = 1.0 - w;
     P.hh = 6.0 * w * (1.0 - w) / (1.0 - 3.0 * w);
     P.bb = (1.0 - w) / (1.0 - 3.0 * w);
@@ -3787,7 +3790,7 @@ lbm_status lbm_set_eos(lbm_ctx* c, int kind, const double* params, int np) {
     }
 
     const double eta0 = p0 / cs2 - r0;  // (p0 / cs2 - (2 + alpha1) rho0) / beta1
-    const double mr[9] = {r0, -2.0 * r0 + 2.0 * eta0, r0 + P.beta2 * eta0, 0, 0, 0, 0, 0, 0};
+    const double mr[9] = {r0, -2.0 * r0 + 2.0 * eta0, r0 + beta2 * eta0, 0, 0, 0, 0, 0, 0};
     const double re = r0 * P.E0, rc = r0 * Cp * T0;
     const double nr[9] = {re, -4.0 * (re - rc) + k.gamma1 * rc, 4.0 * (re - rc) + k.gamma2 * rc, 0, 0, 0, 0, 0, 0};
     host_inverse_moments(mr, c->f_rest);
