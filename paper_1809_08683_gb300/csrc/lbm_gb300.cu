@@ -2842,7 +2842,7 @@ struct lbm_ctx {
     int device = 0;         // device current at lbm_create, which holds the workspace
     BWork* d_bwork = nullptr;
     int n_bwork = 0;
-    int n_node = 0, n_prep = 0;  // CTAs of the node kernels, 0 when the lone lattice steps through strips
+    int n_node = 0, n_prep = 0;  // CTAs of the node kernels, 0 when the lone lattice steps through strips only
     int node_per_cta = 0, prep_per_cta = 0;
     int cluster_ctas = 0;        // CTAs of k_steps_cluster, 0 when the lone lattice is too large for it
     long steps = 0;
@@ -2875,14 +2875,23 @@ constexpr long long kModelMinNodes = 32768;
 // paired ones among them).  Beyond about this many the second read of the DFs,
 // 72 B per node, no longer comes from L2.  us per step of a lone cavity, node
 // kernels and strips: 512^2 16 and 25, 768^2 28 and 37, 1024^2 65 and 49; of a
-// periodic box: 17 and 22, 31 and 40, 77 and 56.  Lattices of up to 160
-// columns, whose warp strips leave more idle, gain up to more nodes: batches
-// of 64 to 128 a side take 61 and 45 us (strips, node kernels) at 0.6M nodes,
-// 132 and 115 at 1.5M, 245 and 249 at 3.1M.
+// periodic box: 17 and 22, 31 and 40, 77 and 56.
+// Lattices of up to 160 columns, whose warp strips leave more idle, gain up to
+// more nodes, but a stepping call starts with a pass for the first step's
+// macros (k_prep), which short calls do not earn back.  Batches of 150^2 (us
+// per step in calls of 50, strips and node kernels): 66 and 45 at 0.65M nodes,
+// 77 and 68 at 1.0M, 88 and 82 at 1.2M, 114 and 125 at 1.8M; a call of one
+// step: 76 and 65, 88 and 97, 97 and 115, 126 and 172.  Lone 160-column
+// channels: 92 and 72 at 1.2M, 111 and 105 at 1.8M, 126 and 121 at 2.1M; one
+// step: 103 and 102, 122 and 146, 138 and 166, so that short calls of a large
+// one step through the strips (at 1.5M nodes calls of two steps 206 and 214
+// us, of four 400 and 392; at 2.4M of four 564 and 593).
 #ifndef LBM_NODE_MAX_FP32
 #define LBM_NODE_MAX_FP32 600000
 #endif
-constexpr long long kNodeMaxNarrow = 2500000;
+constexpr long long kNodeMaxNarrow = 2500000, kNodeMaxNarrowBatch = 900000;
+constexpr long long kNodeShortNodes = 1300000;  // lone narrow lattices from here on step through the strips
+constexpr long kNodeShortSteps = 3;             // in calls of up to this many steps
 constexpr long long kNodeMaxFp32 = LBM_NODE_MAX_FP32;
 
 // The launches of one time step over a set of members: launch groups
@@ -3041,16 +3050,16 @@ bool is_fp32(const lbm_ctx* c) { return c->cfg.precision == LBM_FP32_DEV; }
 // Whether a lattice steps through the node kernels: always when lbm_set_tile
 // chose them; with a default shape, FP64 lattices always, and FP32 lattices
 // while the nodes of their class stepped together (`nodes`: one lattice, or a
-// batch's FP32 members with a default shape) are few enough.  See
-// kNodeMaxFp32.
+// batch's FP32 members with a default shape) are few enough (max_narrow:
+// kNodeMaxNarrow or kNodeMaxNarrowBatch).  See kNodeMaxFp32.
 struct ClassNodes {
     long long narrow = 0, wide = 0;  // default shape: warp strips, others
     void add(const lbm_ctx* c) { (c->pair == 4 ? narrow : wide) += (long long)c->cfg.nx * c->cfg.ny; }
 };
-bool node_kernels(const lbm_ctx* c, const ClassNodes& nodes) {
+bool node_kernels(const lbm_ctx* c, const ClassNodes& nodes, long long max_narrow) {
     if (c->tile_set) return c->pair == 6;
     if (c->cfg.precision == LBM_FP64) return true;
-    return c->pair == 4 ? nodes.narrow <= kNodeMaxNarrow : nodes.wide <= kNodeMaxFp32;
+    return c->pair == 4 ? nodes.narrow <= max_narrow : nodes.wide <= kNodeMaxFp32;
 }
 // Which of them: 0 FP64, 1 FP32, 2 FP32 in pairs (lattices whose strips are paired).
 enum { kNode64 = 0, kNode32 = 1, kNodePair = 2, kNodeKinds = 3 };
@@ -3210,10 +3219,10 @@ void launch_cluster(InstDesc* const* descs, long long nn, int ctas, long nsteps,
 
 lbm_status upload_work(lbm_ctx* c) {
     if (c->d_work) { cudaFree(c->d_work); c->d_work = nullptr; }
-    c->n_node = c->n_prep = c->cluster_ctas = 0;
+    c->n_work = c->n_node = c->n_prep = c->cluster_ctas = 0;
     ClassNodes own;
     own.add(c);
-    if (node_kernels(c, own)) {
+    if (node_kernels(c, own, kNodeMaxNarrow)) {
         // no table: the kernels find a lone lattice's work by themselves
         const int nx = c->cfg.nx, ny = c->cfg.ny, edge = c->h.py ? 0 : 1;
         c->node_per_cta = collide_per_cta(node_kind(c), (long long)nx * ny);
@@ -3221,14 +3230,15 @@ lbm_status upload_work(lbm_ctx* c) {
         c->n_node = node_ctas((long long)(node_kind(c) == kNodePair ? (nx + 1) / 2 : nx) * ny, c->node_per_cta);
         c->n_prep = node_ctas(wall_count(nx, ny, c->h.px, c->h.py), wall_per_cta(prep_threads(is_fp32(c)), c->h.wall_pairs)) + node_ctas((long long)nx * (ny - 2 * edge), c->prep_per_cta);
         c->cluster_ctas = is_fp32(c) ? cluster_ctas_for<float>((long long)nx * ny) : cluster_ctas_for<double>((long long)nx * ny);
-        return LBM_OK;
+        // the strips' table too where short calls take them
+        if (c->tile_set || !is_fp32(c) || c->pair != 4 || (long long)nx * ny < kNodeShortNodes) return LBM_OK;
     }
     c->h_work = make_work(c->cfg, 0, c->bx, c->by, 0, 0);
     split_tail(c->h_work, resident_ctas(variant_index(c->bx, c->pair), is_fp32(c)));
-    c->n_work = (int)c->h_work.size();
     CUDA_TRY(cudaMalloc(&c->d_work, c->h_work.size() * sizeof(Work)));
     CUDA_TRY(cudaMemcpyAsync(c->d_work, c->h_work.data(), c->h_work.size() * sizeof(Work),
                              cudaMemcpyHostToDevice, c->stream));
+    c->n_work = (int)c->h_work.size();
     return LBM_OK;
 }
 
@@ -3968,6 +3978,7 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
     if (nsteps < 0) return fail(LBM_EINVAL, "nsteps < 0");
     if (c->sticky != LBM_OK) return fail(c->sticky, "context is unstable");
     if (nsteps == 0) return LBM_OK;
+    if (!c->n_node && !c->n_work) return fail(LBM_ENOMEM, "no launch table: the last lbm_set_tile or lbm_set_eos failed");
     const long long base = c->steps;
     CUDA_TRY(cudaMemcpyAsync(c->d_counter, &base, sizeof(base), cudaMemcpyHostToDevice, c->stream));
     const bool f32 = is_fp32(c);
@@ -3978,10 +3989,12 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
         c->steps += nsteps;
         return check_launch();
     }
-    launch_prep(f32, c->h.wall_pairs != 0, nullptr, c->n_prep, c->prep_per_cta, c->d_descs, cur_buf(c), 0, nullptr, c->stream);
+    const bool node = c->n_node && !(c->n_work && nsteps <= kNodeShortSteps);
+    if (node)
+        launch_prep(f32, c->h.wall_pairs != 0, nullptr, c->n_prep, c->prep_per_cta, c->d_descs, cur_buf(c), 0, nullptr, c->stream);
     for (long s = 0; s < nsteps; ++s) {
         const int par = (int)((c->steps + s) & 1);
-        if (c->n_node) {
+        if (node) {
             launch_node(node_kind(c), nullptr, c->n_node, c->node_per_cta, c->d_descs, par, c->d_counter, c->stream);
             launch_prep(f32, c->h.wall_pairs != 0, nullptr, c->n_prep, c->prep_per_cta, c->d_descs, par, 1, c->d_counter, c->stream);
         } else if (f32) {
@@ -4369,7 +4382,7 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int n, int graph_steps, lbm_ba
     for (int i = 0; i < n; ++i)
         if (ctxs[i] && !ctxs[i]->tile_set && is_fp32(ctxs[i])) nodes32.add(ctxs[i]);
     std::vector<char> node(n, 0);
-    for (int i = 0; i < n; ++i) node[i] = ctxs[i] && node_kernels(ctxs[i], nodes32);
+    for (int i = 0; i < n; ++i) node[i] = ctxs[i] && node_kernels(ctxs[i], nodes32, kNodeMaxNarrowBatch);
     // rows per run of the members whose shape was not set: the batch length,
     // halved for all of them while the batch fills less than the GPU once
     // (each CTA of a member takes 1 / resident_ctas of the GPU)
