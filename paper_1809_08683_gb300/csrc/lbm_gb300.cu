@@ -4540,6 +4540,8 @@ lbm_status lbm_batch_step(lbm_batch* b, long nsteps) {
     if (b->graph) {
         if (nsteps % b->graph_steps) return fail(LBM_EINVAL, "nsteps must be a multiple of graph_steps");
         batch_launch_first(b, b->set, 0, b->stream);
+        lbm_status st = check_launch();  // without the macros it forms the replays would step on what the field area holds
+        if (st != LBM_OK) return st;
         for (long s = 0; s < nsteps; s += b->graph_steps) CUDA_TRY(cudaGraphLaunch(b->graph, b->stream));
     } else {
         batch_launch_first(b, b->set, (int)(b->steps & 1), b->stream);
