@@ -4014,8 +4014,9 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
         const long long nn = (long long)c->cfg.nx * c->cfg.ny;
         if (f32) launch_cluster<float>(c->d_descs, nn, c->cluster_ctas, nsteps, cur_buf(c), c->d_counter, c->stream);
         else launch_cluster<double>(c->d_descs, nn, c->cluster_ctas, nsteps, cur_buf(c), c->d_counter, c->stream);
-        c->steps += nsteps;
-        return check_launch();
+        lbm_status st = check_launch();
+        if (st == LBM_OK) c->steps += nsteps;
+        return st;
     }
     const bool node = c->n_node && !(c->n_work && nsteps <= kNodeShortSteps);
     if (node)
@@ -4034,7 +4035,7 @@ lbm_status lbm_step(lbm_ctx* c, long nsteps) {
         }
     }
     lbm_status st = check_launch();
-    c->steps += nsteps;
+    if (st == LBM_OK) c->steps += nsteps;
     return st;
 }
 

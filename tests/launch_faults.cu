@@ -97,6 +97,19 @@ int main() {
         EXPECT(lbm_batch_step(&b, 4) == LBM_OK);
         EXPECT(fake::launches == 1 && fake::replays == 2 && b.steps == 4 && c.steps == 4);
     }
+    // a launch of a lone lattice's steps fails: in one cluster, in node kernels
+    for (int cluster = 0; cluster < 2; ++cluster) {
+        lbm_ctx c;
+        context(c);
+        c.n_node = c.n_prep = 1;
+        c.cluster_ctas = cluster;
+        fake::reset(cluster ? 0 : 2, -1);
+        EXPECT(lbm_step(&c, 3) == LBM_ECUDA);
+        EXPECT(c.steps == 0);
+        fake::reset(-1, -1);
+        EXPECT(lbm_step(&c, 3) == LBM_OK);
+        EXPECT(c.steps == 3);
+    }
     if (!failures) std::printf("ok\n");
     return failures ? 1 : 0;
 }
