@@ -4100,8 +4100,9 @@ lbm_status lbm_get_state(lbm_ctx* c, double* f, double* g) {
         CUDA_TRY(cudaMemcpyAsync(host, c->d_stage, n * nn * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         return LBM_OK;
     });
+    const cudaError_t e = cudaStreamSynchronize(c->stream);  // after an error too: copies to f and g may be in flight
     if (st != LBM_OK) return st;
-    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    if (e != cudaSuccess) return fail(LBM_ECUDA, std::string("get_state: ") + cudaGetErrorString(e));
     return LBM_OK;
 }
 
@@ -4116,7 +4117,10 @@ lbm_status lbm_set_state(lbm_ctx* c, const double* f, const double* g) {
         else k_set_planes<double><<<grid, 256, 0, c->stream>>>(c->d_desc, cur_buf(c), q0, r, c->d_stage);
         return check_launch();
     });
-    if (st != LBM_OK) return st;
+    if (st != LBM_OK) {
+        cudaStreamSynchronize(c->stream);  // copies from f and g may be in flight
+        return st;
+    }
     CUDA_TRY(cudaMemsetAsync(c->d_status, 0, 256, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     c->sticky = LBM_OK;

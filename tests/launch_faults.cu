@@ -110,6 +110,16 @@ int main() {
         EXPECT(lbm_step(&c, 3) == LBM_OK);
         EXPECT(c.steps == 3);
     }
+    // state transfers: no copy from or to the caller's arrays is left in flight
+    for (int set = 0; set < 2; ++set)
+        for (int k = 0; k < 4; ++k) {
+            lbm_ctx c;
+            context(c);
+            double f = 0.0, g = 0.0;  // addresses only
+            fake::reset(-1, k);
+            EXPECT((set ? lbm_set_state(&c, &f, &g) : lbm_get_state(&c, &f, &g)) == LBM_ECUDA);
+            EXPECT(fake::copies == k + 1 && fake::syncs_after_copy == 1);
+        }
     if (!failures) std::printf("ok\n");
     return failures ? 1 : 0;
 }

@@ -1,5 +1,6 @@
 """What the library's calls do when a launch or a copy that they issue fails:
-the error comes back from that call and no step is counted.  The CUDA runtime is a fake in the helper (tests/launch_faults.cu),
+the error comes back from that call, no step is counted and no copy stays in
+flight.  The CUDA runtime is a fake in the helper (tests/launch_faults.cu),
 which runs with no GPU visible."""
 import os
 import subprocess
