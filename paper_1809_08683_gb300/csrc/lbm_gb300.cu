@@ -2893,6 +2893,8 @@ constexpr int kModels = 2;  // model classes: lbm::MODEL_ANY, lbm::MODEL_CAVITY
 // cavity model: they are latency-bound, and batches of them (the serving
 // mix) then stay one launch per shape.
 constexpr long long kModelMinNodes = 32768;
+static_assert(ClusterTraits<float>::max_nodes < kModelMinNodes && ClusterTraits<double>::max_nodes < kModelMinNodes,
+              "k_steps_cluster has the generic instance only");
 // Most FP32 nodes that default shapes step through the node kernels, counted
 // over the lattices stepped together whose strips would be block strips (the
 // paired ones among them).  Beyond about this many the second read of the DFs,
