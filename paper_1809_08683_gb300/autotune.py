@@ -1,13 +1,14 @@
-"""Launch-shape autotuner for the fused collide-stream kernel.
+"""Launch-shape autotuner.
 
-The fused kernel gives each CTA a strip of ``bx`` columns (32, 64 or 128
-threads) and a run of ``by`` rows that it sweeps with a three-row ring of
-rho' and p' in shared memory.  Short runs give more CTAs (better SM fill on
-small lattices) but re-read two halo rows per run; long runs amortise the
-halo but may leave SMs idle.  The best shape depends on the lattice shape and
-the precision, so it is measured: every candidate is timed with CUDA events
-on the lattice's own stream, and the winner is cached per
-(precision, nx class, ny class) in a JSON file.
+A fused kernel gives each CTA a strip of ``bx`` columns and a run of ``by``
+rows that it sweeps with a three-row ring of rho' and p' in shared memory.
+Short runs give more CTAs (better SM fill on small lattices) but re-read two
+halo rows per run; long runs amortise the halo but may leave SMs idle.  The
+best shape depends on the lattice shape and the precision, so it is measured:
+every strip shape, and the built-in default (which steps FP64 lattices and
+small FP32 ones through the node kernels), is timed with CUDA events on the
+lattice's own stream, and the winner is cached per (precision, nx class, ny
+class) in a JSON file.
 """
 from __future__ import annotations
 
@@ -22,6 +23,10 @@ _CACHE_PATH = os.environ.get(
 _lock = threading.Lock()
 BX_CANDIDATES = (32, 64, 128)
 BY_CANDIDATES = (4, 8, 16, 32, 64, 128)
+DEFAULT = (0, 0, 0)   # set_tile(0, 0, 0): the built-in default
+# What the cached figures are of.  2: whole steps of plain stepping calls, the
+# default among the shapes.  An entry of another version is measured again.
+_VERSION = 2
 
 
 def size_class(n: int) -> int:
@@ -58,16 +63,15 @@ WARP2_BX_CANDIDATES = (60, 120, 240)
 
 
 def candidates(cfg: dict):
-    """(bx, by, pair) strip shapes worth timing for this lattice: one node per
-    thread in block strips or warp strips for every precision, two nodes per
-    thread for FP32 storage.  A lattice whose shape is not set steps through
-    the node kernels where those are faster (FP64, and small FP32 lattices)."""
+    """(bx, by, pair) shapes worth timing for this lattice: the built-in
+    default, and strips of one node per thread in block strips or warp strips
+    for every precision, two nodes per thread for FP32 storage."""
     shapes = [(bx, 0) for bx in BX_CANDIDATES] + [(bx, 4) for bx in WARP_BX_CANDIDATES]
     if int(cfg.get("precision", 0)) == 1:
         shapes += [(bx, 3) for bx in BX_CANDIDATES]
         shapes += [(bx, pr) for bx in PAIR_BX_CANDIDATES for pr in (1, 2)]
         shapes += [(bx, 5) for bx in WARP2_BX_CANDIDATES]
-    out = []
+    out = [DEFAULT]
     for bx, pr in shapes:
         if bx > 32 and cfg["nx"] <= bx // 2:
             continue
@@ -78,33 +82,46 @@ def candidates(cfg: dict):
     return out
 
 
+def _time_steps(step, stream, steps: int) -> float:
+    """Milliseconds of one stepping call on its stream, between two events
+    around it: events between a step's launches would keep the node kernels
+    from starting early."""
+    import torch
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    a.record(stream)
+    step(steps)
+    b.record(stream)
+    b.synchronize()
+    return a.elapsed_time(b)
+
+
 def measure(cfg: dict, bx: int, by: int, pair: int = 0, steps: int = 20, stream=None) -> float:
-    """MLUPS of whole steps (the fused launch and the wall pass) for one
-    launch shape."""
+    """MLUPS of whole steps of a lone lattice in one launch shape ((0, 0, 0):
+    the built-in default)."""
     lat = lbm.Lattice(cfg, stream=stream)
     lat.set_tile(bx, by, pair)
-    batch = lbm.Batch([lat], graph_steps=0)
-    batch.step_profiled(4)                       # warm-up
-    ms = sum(batch.step_profiled(steps))
-    batch.close()
+    lat.step(4)                                  # warm-up
+    ms = _time_steps(lat.step, lat.stream, steps)
     lat.close()
     return cfg["nx"] * cfg["ny"] * steps / (ms * 1e-3) / 1e6
 
 
 def tune(cfg: dict, steps: int = 20, force: bool = False, stream=None) -> tuple:
-    """Best (bx, by, pair) for this configuration's class, measured on first use."""
+    """Best (bx, by, pair) for this configuration's class, measured on first
+    use; (0, 0, 0), which set_tile takes too, is the built-in default."""
     key = key_for(cfg)
     with _lock:
         cache = _load()
-        if key in cache and not force and len(cache[key]["tile"]) == 3:
-            return tuple(cache[key]["tile"])
+        entry = cache.get(key, {})
+        if not force and entry.get("version") == _VERSION and len(entry["tile"]) == 3:
+            return tuple(entry["tile"])
     results = {}
     for bx, by, pr in candidates(cfg):
         results[(bx, by, pr)] = measure(cfg, bx, by, pr, steps, stream)
     best = max(results, key=results.get)
     with _lock:
         cache = _load()
-        cache[key] = {"tile": list(best), "mlups": results[best],
+        cache[key] = {"version": _VERSION, "tile": list(best), "mlups": results[best],
                       "all": {f"{b[0]}x{b[1]}p{b[2]}": v for b, v in results.items()}}
         _store(cache)
     return best
@@ -124,19 +141,19 @@ BATCH_SHAPES = (None, (128, 16, 1), (128, 24, 1), (128, 32, 1), (128, 48, 1), (2
 
 
 def measure_batch(lattices, shape, steps: int = 10, warmup: int = 3) -> float:
-    """Milliseconds per time step of the whole batch (fused and wall-pass
-    launches, CUDA events) with `shape` applied to every member, or each
-    member's default shape for None.  The shape stays applied."""
+    """Milliseconds per time step of the whole batch (CUDA events around one
+    call) with `shape` applied to every member, or each member's default shape
+    for None.  The shape stays applied."""
     for lat in lattices:
         if shape is None:
             lat.set_tile(0, 0, 0)
         else:
             lat.set_tile(*shape)
     batch = lbm.Batch(lattices, graph_steps=0)
-    batch.step_profiled(warmup)
-    a, b = batch.step_profiled(steps)
+    batch.step(warmup)
+    ms = _time_steps(batch.step, lattices[0].stream, steps)
     batch.close()
-    return (a + b) / steps
+    return ms / steps
 
 
 def tune_batch(lattices, shapes=BATCH_SHAPES, steps: int = 10):

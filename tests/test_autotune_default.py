@@ -1,0 +1,52 @@
+"""The launch-shape tuner can return the built-in default, which is not among
+the strips: the node kernels step through no strip shape, so a tuner that
+chose between strips alone would make such a lattice slower."""
+import json
+
+import pytest
+
+from paper_1809_08683_gb300 import autotune
+from paper_1809_08683_gb300 import workloads as W
+
+
+class FakeLattice:
+    def __init__(self, cfg):
+        self.cfg, self.stream, self.tiles = cfg, None, []
+
+    def set_tile(self, *t):
+        self.tiles.append(t)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_default_is_timed_and_kept_when_fastest(tmp_path, monkeypatch, precision):
+    monkeypatch.setattr(autotune, "_CACHE_PATH", str(tmp_path / "tiles.json"))
+    timed = []
+
+    def measure(cfg, bx, by, pair=0, steps=20, stream=None):
+        timed.append((bx, by, pair))
+        return 2000.0 if (bx, by, pair) == (0, 0, 0) else 1500.0
+
+    monkeypatch.setattr(autotune, "measure", measure)
+    lat = FakeLattice(W.cavity(N=200, precision=precision))
+    autotune.apply([lat])
+    assert timed.count((0, 0, 0)) == 1 and len(timed) > 10
+    assert lat.tiles == [(0, 0, 0)]              # lbm_set_tile's way back to the default
+
+
+def test_entries_of_the_earlier_metric_are_measured_again(tmp_path, monkeypatch):
+    path = tmp_path / "tiles.json"
+    monkeypatch.setattr(autotune, "_CACHE_PATH", str(path))
+    cfg = W.cavity(N=200)
+    path.write_text(json.dumps({autotune.key_for(cfg): {"tile": [64, 8, 0], "mlups": 1.0, "all": {}}}))
+    monkeypatch.setattr(autotune, "measure", lambda cfg, bx, by, pair=0, steps=20, stream=None: 100.0 - by)
+    assert autotune.tune(cfg) == (0, 0, 0)
+    assert autotune.tune(cfg) == (0, 0, 0) and json.loads(path.read_text())[autotune.key_for(cfg)]["tile"] == [0, 0, 0]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", [0, 1])
+def test_tuned_lattice_keeps_the_node_kernels(tmp_path, monkeypatch, precision):
+    """256^2 takes 70 us per step (FP64) and 9 (FP32) in the node kernels, 95
+    and 13 in the best strips."""
+    monkeypatch.setattr(autotune, "_CACHE_PATH", str(tmp_path / "tiles.json"))
+    assert autotune.tune(W.cavity(N=256, Ra=1e5, eps=0.5, precision=precision)) == (0, 0, 0)
