@@ -111,8 +111,6 @@ def workload(name, precision):
     return cfgs, {"workload": "poiseuille_4x128_cubic", "precision": "fp32_dev" if p else "fp64"}, 1000
 
 
-KERNEL_OF_PAIR = {0: "k_collide_stream", 1: "k_collide_pair", 2: "k_collide_pair", 3: "k_collide_stream",
-                  4: "k_collide_warp", 5: "k_collide_warp2", 6: "k_collide_node"}
 KERNEL_SOURCES = ("lbm_gb300.cu", "lbm_node.cuh", "lbm_f2.cuh")
 
 
@@ -615,10 +613,8 @@ def main():
     avg_collide_ms = t_collide / psteps
     alg_bytes = nodes * BYTES_PER_NODE[prec]
     achieved = alg_bytes / (avg_collide_ms * 1e-3) / 1e9
-    kernels = sorted({KERNEL_OF_PAIR[lat.tile()[2]] for lat in lats})
-    kernel = "+".join(kernels)
-    n_collide_launches = len({(lat.tile()[0], lat.tile()[2], lat.cfg.get("precision", 0)) for lat in lats})
-    gpu_launches = steps_total * (n_collide_launches + 1)
+    kernel, per_step, per_call = batch.kernels()
+    gpu_launches = steps_total * per_step + args.steps * per_call
     traffic = read_traffic(desc["workload"], kernel)
 
     # end to end through the public API with host buffers

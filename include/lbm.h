@@ -264,9 +264,18 @@ lbm_status lbm_batch_step(lbm_batch* b, long nsteps);
 lbm_status lbm_batch_destroy(lbm_batch* b);     /* NULL-safe */
 
 /* Same as lbm_batch_step without the graph, with CUDA events recorded on the
- * batch stream around each step's fused launches and wall-pass launches;
+ * batch stream around each step's fused launches and wall-pass launches (node
+ * kernels: collision, and wall nodes with the macros);
  * *ms_collide and *ms_wall receive their summed device times.  Synchronises. */
 lbm_status lbm_batch_step_profiled(lbm_batch* b, long nsteps, double* ms_collide, double* ms_wall);
+
+/* What lbm_batch_step launches, for reports: the names of the kernels that
+ * collide and push the members' nodes, joined by '+' in alphabetical order,
+ * into names (host, bytes long, cut and terminated if short), the launches of
+ * one time step into *per_step and those at the start of every call into
+ * *per_call (each may be NULL).  lbm_get_tile reports a member's shape, which
+ * does not say whether its node kernels run. */
+lbm_status lbm_batch_kernels(const lbm_batch* b, char* names, size_t bytes, int* per_step, int* per_call);
 
 /* lbm_diagnostics for every member of a batch in one pass: one launch per
  * storage precision over all members, one copy back and one

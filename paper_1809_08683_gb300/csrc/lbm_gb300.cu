@@ -4605,6 +4605,36 @@ lbm_status lbm_batch_step_profiled(lbm_batch* b, long nsteps, double* ms_collide
     return LBM_OK;
 }
 
+lbm_status lbm_batch_kernels(const lbm_batch* b, char* names, size_t bytes, int* per_step, int* per_call) {
+    if (!b) return fail(LBM_EINVAL, "null batch");
+    static const char* const kOfPair[] = {"k_collide_stream", "k_collide_pair", "k_collide_pair", "k_collide_stream",
+                                          "k_collide_warp", "k_collide_warp2"};
+    static const char* const kOfKind[kNodeKinds] = {"k_collide_node", "k_collide_node", "k_collide_node2"};
+    const LaunchSet& ls = b->set;
+    std::vector<std::string> found;
+    int step = 0, call = 0;
+    auto add = [&](const char* name) {
+        ++step;
+        if (std::find(found.begin(), found.end(), name) == found.end()) found.push_back(name);
+    };
+    for (int k = 0; k < kNodeKinds; ++k)
+        if (ls.n_cnt[k]) add(kOfKind[k]);
+    for (int pr = 0; pr < 2; ++pr) {
+        for (int vi = 0; vi < kVariants; ++vi)
+            for (int mc = 0; mc < kModels; ++mc)
+                if (ls.w_cnt[pr][vi][mc]) add(kOfPair[kVariantPair[vi]]);
+        step += (ls.b_cnt[pr] ? 1 : 0) + (ls.p_cnt[pr] ? 1 : 0);
+        call += ls.p_cnt[pr] ? 1 : 0;
+    }
+    std::sort(found.begin(), found.end());
+    std::string all;
+    for (const std::string& f : found) all += (all.empty() ? "" : "+") + f;
+    if (names && bytes) std::snprintf(names, bytes, "%s", all.c_str());
+    if (per_step) *per_step = step;
+    if (per_call) *per_call = call;
+    return LBM_OK;
+}
+
 lbm_status lbm_batch_diagnostics(lbm_batch* b, int snapshot, double* out8n, int* member_status) {
     if (!b || !out8n) return fail(LBM_EINVAL, "bad batch diagnostics arguments");
     const int n = (int)b->ctxs.size();

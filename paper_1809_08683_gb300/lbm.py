@@ -75,7 +75,7 @@ EXPORTS = ("lbm_workspace_bytes", "lbm_create", "lbm_set_eos", "lbm_step", "lbm_
            "lbm_last_error", "lbm_batch_create", "lbm_batch_step", "lbm_batch_step_profiled",
            "lbm_batch_destroy", "lbm_conserved_sums_static", "lbm_set_rounding", "lbm_copy_state",
            "lbm_wait_selftest", "lbm_batch_diagnostics", "lbm_batch_add", "lbm_batch_remove",
-           "lbm_peak_rates", "lbm_batch_init_macros", "lbm_batch_macros")
+           "lbm_peak_rates", "lbm_batch_init_macros", "lbm_batch_macros", "lbm_batch_kernels")
 
 
 def load(path: str | None = None):
@@ -123,6 +123,7 @@ def load(path: str | None = None):
         L.lbm_batch_remove.argtypes = [vp, vp]
         L.lbm_batch_init_macros.argtypes = [vp, P(dp), P(dp), P(dp), P(dp)]
         L.lbm_batch_macros.argtypes = [vp, P(dp), P(dp), P(dp), P(dp), P(dp), P(C.c_int)]
+        L.lbm_batch_kernels.argtypes = [vp, C.c_char_p, C.c_size_t, P(i), P(i)]
         _lib = L
         return L
 
@@ -337,6 +338,13 @@ class Batch:
         a, b = C.c_double(), C.c_double()
         _check(self.L, self.L.lbm_batch_step_profiled(self.h, int(n), C.byref(a), C.byref(b)))
         return a.value, b.value
+
+    def kernels(self):
+        """What step() launches: (names of the collision kernels joined by
+        '+', launches per time step, launches at the start of a call)."""
+        names, a, b = C.create_string_buffer(256), C.c_int(), C.c_int()
+        _check(self.L, self.L.lbm_batch_kernels(self.h, names, 256, C.byref(a), C.byref(b)))
+        return names.value.decode(), a.value, b.value
 
     def add(self, lattice):
         """Append a member (launch tables and graph rebuilt)."""
