@@ -30,8 +30,8 @@ Fields of the JSON line (rank 0):
   serving   a Poisson stream of cavity and channel solves to residual 1e-7
             through the continuous-batching server; a subset solved four
             ways (batched or one at a time, FP32 then FP64 or FP64 only)
-  fp64_path the FP64-storage kernel on a 2048^2 cavity against the probed
-            FP64 FMA rate
+  fp64_path whole steps of a 2048^2 FP64 cavity in the default launch shape
+            against the probed FP64 FMA rate
   cpu_baseline  the FP64 CPU oracle on a bounded sample (rank 0, N = 1)
 `--impl reference` times that oracle alone (the reference arm).
 Multi-GPU: instances are independent, so each rank advances its own copy of
@@ -387,39 +387,40 @@ def table2_run(Ra, steps, every=20_000):
             "series": [[r[0], round(r[1], 5), round(r[2], 5), round(r[3], 6)] for r in rec[::5]]}
 
 
-# FP64 operations per node update of the heated-cavity model, counted by
-# instantiating the node templates with an operation-counting number type:
-# 308 additions, 289 multiplications, 10 divisions, 1 square root, and
-# about 36 for the gradient stencil.
-FP64_OPS_PER_NODE = 644
+# FP64 instructions per inner node and time step of the heated-cavity model:
+# 317 of the collision (smsp__inst_executed_pipe_fp64 of a 512^2 cavity over
+# its nodes) and 44 of the macros.
+FP64_INSTRUCTIONS_PER_NODE = 361
 
 
 def fp64_path(n_side=2048, steps=10):
-    """The FP64-storage fused kernel on an n_side^2 heated cavity (Ra =
-    1e8, eps = 0.6, block strips): per-step time and counted FP64 operation
-    rate against the device's probed FP64 FMA rate, which bounds it."""
+    """Whole time steps of an n_side^2 FP64 heated cavity (Ra = 1e8, eps =
+    0.6) in the default launch shape, and the rate of the FP64 instructions
+    they cannot do without against the device's probed FP64 FMA rate, which
+    bounds it."""
     import torch
     from paper_1809_08683_gb300 import lbm
     st = torch.cuda.Stream()
     rates = lbm.peak_rates(st)
     cfg = W.cavity(N=n_side, Ra=1e8, eps=0.6, precision=0)
-    out = {"workload": f"cavity_{n_side}x{n_side}_Ra1e8_eps0.6_fp64", "rates": rates,
-           "ops_per_node": FP64_OPS_PER_NODE}
     with torch.cuda.stream(st):
         lat = lbm.Lattice(cfg, stream=st)
-    for name, tile in (("native_fp64", (128, 8, 0)),):
-        lat.set_tile(*tile)
-        b = lbm.Batch([lat], graph_steps=0)
-        b.step_profiled(3)
-        ms, _ = b.step_profiled(steps)
-        b.close()
-        mlups = n_side * n_side * steps / (ms * 1e-3) / 1e6
-        out[name] = {"tile": list(tile), "fused_ms_per_step": ms / steps, "mlups": mlups,
-                     "counted_gflops": mlups * FP64_OPS_PER_NODE / 1e3}
+    b = lbm.Batch([lat], graph_steps=0)
+    b.step(3)
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    e0.record(st)
+    b.step(steps)
+    e1.record(st)
+    e1.synchronize()
+    ms = e0.elapsed_time(e1)
+    kernel = b.kernels()[0]
+    b.close()
     lat.close()
-    # FP64 FMA counts two operations
-    out["native_fp64"]["frac_of_fp64_peak"] = out["native_fp64"]["counted_gflops"] * 1e9 / (2 * rates["fp64_fma_per_s"])
-    return out
+    mlups = n_side * n_side * steps / (ms * 1e-3) / 1e6
+    issued = mlups * 1e6 * FP64_INSTRUCTIONS_PER_NODE
+    return {"workload": f"cavity_{n_side}x{n_side}_Ra1e8_eps0.6_fp64", "rates": rates, "kernel": kernel,
+            "ms_per_step": ms / steps, "mlups": mlups, "fp64_instructions_per_node": FP64_INSTRUCTIONS_PER_NODE,
+            "fp64_instructions_per_s": issued, "frac_of_fp64_rate": issued / rates["fp64_fma_per_s"]}
 
 
 def steady_sweep_subset(tol=1e-5, max_side=256, deadline_s=None):
