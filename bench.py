@@ -129,9 +129,15 @@ def kernel_source_hash():
     return h.hexdigest()
 
 
-def read_traffic(workload, kernel):
+def shape_name(shape):
+    """A launch shape in reports: bx,by,pair, or "default" for None."""
+    return "default" if shape is None else ",".join(map(str, shape))
+
+
+def read_traffic(workload, kernel, shape=None):
     """DRAM bytes per fused launch from the committed ncu summary of this
-    workload, or None when there is none or the kernels changed since."""
+    workload in this launch shape (None: the default), or None when there is
+    none or the kernels changed since."""
     path = os.path.join(ROOT, "profiles", f"traffic_{workload}.txt")
     try:
         kv = {}
@@ -140,7 +146,8 @@ def read_traffic(workload, kernel):
                 if "=" in line and not line.lstrip().startswith("#"):
                     k, v = line.split("=", 1)
                     kv[k.strip()] = v.strip()
-        if kv.get("kernel") != kernel or kv.get("source_sha256") != kernel_source_hash():
+        if (kv.get("kernel"), kv.get("shape", "default"), kv.get("source_sha256")) != (kernel, shape_name(shape),
+                                                                            kernel_source_hash()):
             return None
         return float(kv["dram_bytes_per_launch"])
     except Exception:
@@ -553,16 +560,17 @@ def main():
     stream = torch.cuda.Stream(device=dev)
     with torch.cuda.stream(stream):
         lats = [lbm.Lattice(c, stream=stream, device=dev) for c in cfgs]
-    tuned = None
+    tuned = shape = None
     if args.tile:
         t = [int(v) for v in args.tile.split(",")]
+        shape = (t[0], t[1], t[2] if len(t) > 2 else 0)
         for lat in lats:
-            lat.set_tile(t[0], t[1], t[2] if len(t) > 2 else 0)
+            lat.set_tile(*shape)
     elif not args.no_tune:
-        best, res = autotune.tune_batch(lats)
-        tuned = {"pick": None if best is None else list(best), "ms_per_step": {
-            ("default" if k is None else ",".join(map(str, k))): v for k, v in res.items()},
-            "default_ms": res[None], "pick_ms": res[best]}
+        shape, res = autotune.tune_batch(lats)
+        tuned = {"pick": None if shape is None else list(shape),
+                 "ms_per_step": {shape_name(k): v for k, v in res.items()},
+                 "default_ms": res[None], "pick_ms": res[shape]}
     nodes = sum(c["nx"] * c["ny"] for c in cfgs)
     prec = int(cfgs[0].get("precision", 0))
     graph_steps = chunk if chunk % 2 == 0 else 0
@@ -616,7 +624,7 @@ def main():
     achieved = alg_bytes / (avg_collide_ms * 1e-3) / 1e9
     kernel, per_step, per_call = batch.kernels()
     gpu_launches = steps_total * per_step + args.steps * per_call
-    traffic = read_traffic(desc["workload"], kernel)
+    traffic = read_traffic(desc["workload"], kernel, shape)
 
     # end to end through the public API with host buffers
     e2e = None
