@@ -6,7 +6,8 @@
 // arithmetic of lbm_node.cuh is instantiated with R = f2 unchanged.  Every
 // lane rounds exactly like the scalar FP32 operation it replaces, and the
 // node arithmetic names each fused multiply-add (mad) while the compiler's
-// own contraction is off, so a lane has the bits of the scalar instance.
+// own contraction is off; what the assembler contracts in the packed form
+// all the same is named in lbm_node.cuh.
 #pragma once
 
 #include <cuda_runtime.h>

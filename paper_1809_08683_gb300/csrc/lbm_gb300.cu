@@ -23,8 +23,8 @@
 // strips (k_collide_warp2); default_shape picks one per lattice and
 // lbm_set_tile selects any other.
 //
-// FP64 lattices, and FP32 ones of few nodes, step with the same bits through
-// two other kernels (node_kernels says when):
+// FP64 lattices, and FP32 ones of few nodes, step with the bits of their strips
+// through two other kernels (node_kernels says when):
 //   k_prep           : rebuilds the wall nodes and writes every node's
 //                      macros to a field array;
 //   k_collide_node   : collides and pushes one node per thread in row-major

@@ -17,11 +17,15 @@
 //  M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4).
 //
 // Every fused multiply-add is written as mad() and the library is compiled
-// without the compiler's own contraction (-fmad=false), so a node's bits
-// depend on its inputs alone: all kernels, scalar or packed, that update a
-// lattice give the same state.  A product with a literal constant that meets
-// an addition is always a mad(): the assembler contracts the packed form of
-// that pair of instructions all the same.
+// without the compiler's own contraction (-fmad=false), so that a node's bits
+// do not depend on the kernel.  One set of bits: the one-node kernels of one
+// model class (block strips, warp strips, node kernels, the cluster kernel);
+// and the paired block strips with their node kernel.  The packed kernels draw
+// one random number per two nodes; with stores rounded to nearest they give
+// the one-node bits too in MODEL_ANY, where a product with a literal constant
+// that meets an addition is always a mad() (the assembler contracts the packed
+// form of that pair of instructions all the same).  In MODEL_CAVITY it
+// contracts more, and the two agree to rounding.
 #pragma once
 
 #include <cmath>
@@ -144,9 +148,9 @@ enum { EOS_DECOUPLING = 0, EOS_IDEAL = 1, EOS_CS = 2, EOS_CUBIC = 3 };
 // mode and the corrections flag from the parameters at run time.
 // MODEL_CAVITY fixes the heated-cavity model at compile time (Sutherland
 // viscosity, F = rho g with vertical g, corrections on) and keeps only the
-// ideal-gas and cubic EOS, chosen at run time.  The arithmetic is the same;
-// a fixed model drops the branches and the code of the others, and the
-// terms of F_x = 0.
+// ideal-gas and cubic EOS, chosen at run time.  A fixed model drops the
+// branches and the code of the others, and the terms of F_x = 0, without
+// which some sums are formed in another order: the classes agree to rounding.
 enum { MODEL_ANY = 0, MODEL_CAVITY = 1 };
 template <int MC, typename R>
 LBM_HD int visc_law(const Params<R>& P) { return MC != MODEL_ANY ? 2 : P.visc; }
