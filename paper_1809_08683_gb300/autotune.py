@@ -27,6 +27,10 @@ DEFAULT = (0, 0, 0)   # set_tile(0, 0, 0): the built-in default
 # What the cached figures are of.  2: whole steps of plain stepping calls, the
 # default among the shapes.  An entry of another version is measured again.
 _VERSION = 2
+# A shape replaces the default only when it is faster by more than the timings
+# of one shape differ.  (The default of a batch can be a listed shape, and set
+# by name that would no longer follow the members.)
+_GAIN = 1.005
 
 
 def size_class(n: int) -> int:
@@ -119,6 +123,8 @@ def tune(cfg: dict, steps: int = 20, force: bool = False, stream=None) -> tuple:
     for bx, by, pr in candidates(cfg):
         results[(bx, by, pr)] = measure(cfg, bx, by, pr, steps, stream)
     best = max(results, key=results.get)
+    if results[best] <= _GAIN * results[DEFAULT]:
+        best = DEFAULT
     with _lock:
         cache = _load()
         cache[key] = {"version": _VERSION, "tile": list(best), "mlups": results[best],
@@ -167,6 +173,8 @@ def tune_batch(lattices, shapes=BATCH_SHAPES, steps: int = 10):
                 continue
         results[shape] = measure_batch(lattices, shape, steps)
     best = min(results, key=results.get)
+    if None in results and results[None] <= _GAIN * results[best]:
+        best = None
     for lat in lattices:
         if best is None:
             lat.set_tile(0, 0, 0)

@@ -43,6 +43,22 @@ def test_entries_of_the_earlier_metric_are_measured_again(tmp_path, monkeypatch)
     assert autotune.tune(cfg) == (0, 0, 0) and json.loads(path.read_text())[autotune.key_for(cfg)]["tile"] == [0, 0, 0]
 
 
+def test_a_tie_leaves_the_default(tmp_path, monkeypatch):
+    monkeypatch.setattr(autotune, "_CACHE_PATH", str(tmp_path / "tiles.json"))
+    gain = {(64, 8, 0): 1.004}
+    monkeypatch.setattr(autotune, "measure", lambda cfg, bx, by, pair=0, steps=20, stream=None:
+                        1000.0 * gain.get((bx, by, pair), 1.0))
+    assert autotune.tune(W.cavity(N=300)) == (0, 0, 0)
+    gain[(64, 8, 0)] = 1.02
+    assert autotune.tune(W.cavity(N=300), force=True) == (64, 8, 0)
+    ms = {(128, 32, 1): 1.1000, None: 1.1002}
+    monkeypatch.setattr(autotune, "measure_batch", lambda lats, shape, steps=10, warmup=3: ms.get(shape, 1.2))
+    lat = FakeLattice({"precision": 1})
+    assert autotune.tune_batch([lat])[0] is None and lat.tiles == [(0, 0, 0)]
+    ms[(128, 32, 1)] = 1.08
+    assert autotune.tune_batch([lat])[0] == (128, 32, 1)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("precision", [0, 1])
 def test_tuned_lattice_keeps_the_node_kernels(tmp_path, monkeypatch, precision):
