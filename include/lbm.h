@@ -226,8 +226,9 @@ lbm_status lbm_set_tile(lbm_ctx* ctx, int bx, int by, int pair);
  * While a shape is the default, FP64 lattices, and FP32 lattices of few
  * nodes (alone, or the FP32 members of a batch together: 600,000, or of up
  * to 160 columns 900,000 in a batch and 2,500,000 alone, there from
- * 1,300,000 on only in calls of more than three steps), step through node
- * kernels that give the bits of that shape, which stays what is reported. */
+ * 1,300,000 on mostly in calls of more than three steps only), step through
+ * node kernels that give the bits of that shape, which stays what is
+ * reported. */
 lbm_status lbm_get_tile(const lbm_ctx* ctx, int* bx, int* by, int* pair);
 
 /* Steps taken since the last (re)initialisation. */

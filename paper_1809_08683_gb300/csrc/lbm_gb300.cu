@@ -2838,7 +2838,8 @@ static_assert(ClusterTraits<float>::max_nodes < kModelMinNodes && ClusterTraits<
 // channels: 92 and 72 at 1.2M, 111 and 105 at 1.8M, 126 and 121 at 2.1M; one
 // step: 103 and 102, 122 and 146, 138 and 166, so that short calls of a large
 // one step through the strips (at 1.5M nodes calls of two steps 206 and 214
-// us, of four 400 and 392; at 2.4M of four 564 and 593).
+// us, of four 400 and 392; at 2.4M of four 564 and 593; but 64 x 30,000, whose
+// three strips are 90 columns wide, in calls of three 477 and 394).
 #ifndef LBM_NODE_MAX_FP32
 #define LBM_NODE_MAX_FP32 600000
 #endif
@@ -3188,8 +3189,10 @@ lbm_status upload_work(lbm_ctx* c) {
         c->n_node = node_ctas((long long)(node_kind(c) == kNodePair ? (nx + 1) / 2 : nx) * ny, c->node_per_cta);
         c->n_prep = node_ctas(wall_count(nx, ny, c->h.px, c->h.py), wall_per_cta(prep_threads(is_fp32(c)), c->h.wall_pairs)) + node_ctas((long long)nx * (ny - 2 * edge), c->prep_per_cta);
         c->cluster_ctas = is_fp32(c) ? cluster_ctas_for<float>((long long)nx * ny) : cluster_ctas_for<double>((long long)nx * ny);
-        // the strips' table too where short calls take them
-        if (c->tile_set || !is_fp32(c) || c->pair != 4 || (long long)nx * ny < kNodeShortNodes) return LBM_OK;
+        // the strips' table too where short calls take them: not where the strips
+        // of 30 columns are more than 1.25 times as wide as the lattice
+        const bool wasteful = 4 * ((nx + 29) / 30) * 30 > 5 * nx;
+        if (c->tile_set || !is_fp32(c) || c->pair != 4 || (long long)nx * ny < kNodeShortNodes || wasteful) return LBM_OK;
     }
     c->h_work = make_work(c->cfg, 0, c->bx, c->by, 0, 0);
     split_tail(c->h_work, resident_ctas(variant_index(c->bx, c->pair), is_fp32(c)));
