@@ -20,12 +20,11 @@
 // without the compiler's own contraction (-fmad=false), so that a node's bits
 // do not depend on the kernel.  One set of bits: the one-node kernels of one
 // model class (block strips, warp strips, node kernels, the cluster kernel);
-// and the paired block strips with their node kernel.  The packed kernels draw
-// one random number per two nodes; with stores rounded to nearest they give
-// the one-node bits too in MODEL_ANY, where a product with a literal constant
-// that meets an addition is always a mad() (the assembler contracts the packed
-// form of that pair of instructions all the same).  In MODEL_CAVITY it
-// contracts more, and the two agree to rounding.
+// and the paired block strips with their node kernel.  The packed kernels
+// agree with the one-node kernels to rounding: they draw one random number per
+// two nodes, and the assembler contracts some packed products that meet an
+// addition all the same (those with a literal constant always, which is why
+// such a product is a mad() throughout).
 #pragma once
 
 #include <cmath>
