@@ -3039,7 +3039,7 @@ int prep_per_cta(bool fp32, long long nodes) {
 // and give small lattices more CTAs.  Wider FP32 lattices of the heated-
 // cavity model class take paired block strips of 128 columns (pair 1): two
 // nodes per thread in packed FP32 halve the arithmetic's issue slots (96-
-// cavity batch: 1.112 ms per step against 1.285 ms for block strips).  All
+// cavity batch: 1.109 ms per step against 1.300 ms for block strips).  All
 // others take block strips of 128 columns (pair 0), in FP64 too.  The model class is known
 // once the EOS is set, so lbm_set_eos applies the shape.
 void default_shape(const lbm_config& c, int mc, int& bx, int& pair) {
