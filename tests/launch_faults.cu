@@ -110,6 +110,14 @@ int main() {
         EXPECT(lbm_step(&c, 3) == LBM_OK);
         EXPECT(c.steps == 3);
     }
+    // without a launch table (lbm_set_tile or lbm_set_eos ran out of memory) nothing is launched
+    {
+        lbm_ctx c;
+        context(c);
+        fake::reset(-1, -1);
+        EXPECT(lbm_step(&c, 2) == LBM_ENOMEM);
+        EXPECT(fake::launches == 0 && c.steps == 0);
+    }
     // state transfers: no copy from or to the caller's arrays is left in flight
     for (int set = 0; set < 2; ++set)
         for (int k = 0; k < 4; ++k) {
